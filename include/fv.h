@@ -404,7 +404,11 @@ int fv_mesh_debug_set_index(fv_mesh* mesh, int32_t table, int64_t cell, int32_t 
  *            step produced a bad state.  If NULL nothing is synchronised; use
  *            fv_mesh_status to collect the outcome later.
  * The step loop runs as captured CUDA graphs of one fused kernel per step;
- * the first call with a new (U, scheme, cfl, t_stop, closure) captures them. */
+ * the first call with a new (U, scheme, cfl, t_stop, closure) captures them.
+ * FV_F32 meshes of up to 12,288 cells whose kernel shape was not chosen
+ * (fv_mesh_set_variant) and that step without a closure run the whole loop in
+ * one launch on one thread-block cluster instead (also with two steps per
+ * launch, when their tile size was left to the library); same bits. */
 int fv_step(fv_mesh* mesh, void* U, int64_t nsteps, double cfl, double t_stop, int32_t scheme,
             const fv_closure* closure, void* stream, double* t_advanced);
 

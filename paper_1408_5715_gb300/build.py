@@ -25,7 +25,7 @@ BUILD_DIR_DEBUG = os.path.join(PKG, "_build_debug")
 SOURCES = ["host_mesh.cpp", "renumber.cpp", "partition.cpp", "tiles.cpp", "vertex_geom.cpp",
            "kernels.cu", "tma_step.cu",
            "tile_step.cu",
-           "pair_step.cu", "closure.cu",
+           "pair_step.cu", "loop_step.cu", "closure.cu",
            "capi.cu", "totals_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

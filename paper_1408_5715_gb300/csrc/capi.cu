@@ -63,6 +63,19 @@ void dev_free(T*& p) {
 constexpr int64_t kGraphSteps = 96;
 constexpr int kBatchTile = 1024;  // cells per tile of the batched shared-memory shape
 
+// The resident loop: cells per block at least (smaller tiles only add blocks
+// to wait for), steps per launch at most (bounds the time of one launch) and
+// tries of a wait (about a second).  It takes meshes of up to kLoopMaxTiles *
+// kLoopMaxTile = 12,288 cells, one per thread.  Measured (us per step, forward
+// Euler, compensated; shape 1 / tiles of 128 / loop): 1,024 cells 2.4 / 2.5 /
+// 0.93, 4,096 2.8 / 2.5 / 0.99, 8,192 2.8 / 2.5 / 1.5; two cells per thread
+// lose their lead (16,200 cells 2.9 / 2.5 / 2.7, 32,768 2.9 / 2.7 / 4.3): 16
+// SMs then compute longer than a launch on all of them takes.
+constexpr int64_t kLoopMinTile = 64;
+constexpr int64_t kLoopMaxCells = (int64_t)fv::kLoopMaxTiles * fv::kLoopMaxTile;
+constexpr int64_t kLoopSteps = 4096;
+constexpr unsigned kLoopPolls = 1u << 20;
+
 }  // namespace
 
 namespace fv {
@@ -147,6 +160,20 @@ struct fv_mesh {
   fv::FaceRec* d_faces = nullptr;
   int64_t n_faces = 0;
   float* d_scale = nullptr;
+  // the resident loop (loop_step.cu): tiles of the whole-loop kernel, built
+  // with the device arrays when one cluster holds the mesh (loop_tiles = 0: not).
+  // It runs where no shape was chosen, or the autotuner found it faster than
+  // every shape (loop_wanted).
+  bool loop_wanted = true;
+  int loop_tile = 0, loop_tiles = 0, loop_cap = 0;
+  unsigned char* d_loop = nullptr;  // holds the arrays below
+  float4* loop_geom = nullptr;
+  uint2* loop_ln = nullptr;
+  int* loop_ord = nullptr;
+  int4* loop_info = nullptr;
+  int* loop_ring = nullptr;       // cells of the tiles' rings
+  unsigned* loop_push = nullptr;  // where the tiles' edge cells go
+  bool pair_default = true;  // fv_mesh_set_blocking left the tile size to the library
   unsigned wait_limit = fv::kDefaultWaitLimit;  // bounded device waits (variant 5)
   fv::LoopScalars* d_scal = nullptr;
   double* d_partials = nullptr;
@@ -207,10 +234,16 @@ struct fv_mesh {
     n_faces = 0;
   }
 
+  void free_loop() {
+    dev_free(d_loop);
+    loop_tile = loop_tiles = loop_cap = 0;
+  }
+
   void free_device() {
     drop_graph();
     free_tiles();
     free_faces();
+    free_loop();
     dev_free(d_nbr);
     dev_free(d_geom);
     dev_free(d_vol);
@@ -353,6 +386,56 @@ size_t pair_smem(const fv_mesh* m) {
   return fv::pair_smem_bytes(m->p_e_cap, m->p_t1_cap, m->tiles_built, m->pair_staged != 0);
 }
 
+// Tiles of the resident loop for a small FP32 mesh, up to kLoopMaxTiles of
+// them; other meshes run a launch per step.
+void build_loop(fv_mesh* m, cudaStream_t s) {
+  m->free_loop();
+  const int64_t n = m->h.n;
+  if (m->f64() || n < 1 || n > kLoopMaxCells) return;
+  const int64_t tile = std::max(kLoopMinTile, (n + fv::kLoopMaxTiles - 1) / fv::kLoopMaxTiles);
+  const fv::LoopTiles L = fv::build_loop_tiles(m->h, (int32_t)tile);
+  // the device can hold the cluster, with every kind of remainder
+  fv::LoopArgs a{};
+  a.tile = L.tile;
+  a.n_tiles = L.n_tiles;
+  a.cap = L.cap;
+  for (bool rk2 : {false, true}) {
+    int clusters = 0;
+    if (fv::loop_clusters(a, rk2, true, &clusters) != cudaSuccess || clusters < 1) {
+      cudaGetLastError();
+      return;
+    }
+  }
+  // one allocation and one copy: the geometry in the loop's order, then the tables
+  const size_t geom_bytes = (size_t)n * 2 * sizeof(float4);
+  std::vector<unsigned char> host;
+  auto put = [&](const auto& v, size_t align, size_t at_least) {
+    host.resize((host.size() + align - 1) / align * align);
+    const size_t at = host.size(), bytes = v.size() * sizeof(v[0]);
+    host.resize(at + std::max(bytes, at_least));
+    if (bytes) std::memcpy(host.data() + at, v.data(), bytes);
+    return geom_bytes + at;
+  };
+  const size_t info = put(L.info, 16, fv::kLoopMaxTiles * sizeof(int4));
+  const size_t ln = put(L.cell_ln, 8, 0), ord = put(L.ord, 4, 0);
+  const size_t ring = put(L.ring_id, 4, 4), push = put(L.push, 4, 4);
+  FV_CUDA(cudaMalloc((void**)&m->d_loop, geom_bytes + host.size()));
+  FV_CUDA(cudaMemcpyAsync(m->d_loop + geom_bytes, host.data(), host.size(), cudaMemcpyHostToDevice,
+                          s));
+  m->loop_geom = reinterpret_cast<float4*>(m->d_loop);
+  m->loop_info = reinterpret_cast<int4*>(m->d_loop + info);
+  m->loop_ln = reinterpret_cast<uint2*>(m->d_loop + ln);
+  m->loop_ord = reinterpret_cast<int*>(m->d_loop + ord);
+  m->loop_ring = reinterpret_cast<int*>(m->d_loop + ring);
+  m->loop_push = reinterpret_cast<unsigned*>(m->d_loop + push);
+  FV_CUDA(fv::launch_loop_geometry(static_cast<const float4*>(m->d_geom), m->loop_ord, (int)n,
+                                   m->loop_geom, s));
+  FV_CUDA(cudaStreamSynchronize(s));  // host is a local staging buffer
+  m->loop_tile = L.tile;
+  m->loop_tiles = L.n_tiles;
+  m->loop_cap = L.cap;
+}
+
 void ensure_device(fv_mesh* m, cudaStream_t s) {
   int dev = 0;
   FV_CUDA(cudaGetDevice(&dev));
@@ -394,6 +477,7 @@ void ensure_device(fv_mesh* m, cudaStream_t s) {
     FV_CUDA(cudaMemcpyAsync(m->d_vol, m->h.vol.data(), n * sizeof(double), cudaMemcpyHostToDevice,
                             s));
     FV_CUDA(cudaStreamSynchronize(s));  // lay is a local staging buffer
+    build_loop(m, s);
   }
   FV_CUDA(cudaStreamSynchronize(s));
   m->device = dev;
@@ -597,6 +681,52 @@ void enqueue_launches(fv_mesh* m, void* U, int64_t j0, int64_t launches, double 
     enqueue_steps(m, U, j0, launches, cfl, t_stop, scheme, s, cl);
 }
 
+// Whether fv_step runs the resident loop: the mesh has its tiles, nothing
+// asks for a kernel shape of its own, and with two steps per launch the tile
+// size was left to the library.
+bool uses_loop(const fv_mesh* m, const fv_closure* cl) {
+  if (m->loop_tiles == 0 || cl || m->vertex_tiles()) return false;
+  return m->blocking == 2 ? m->pair_default : m->loop_wanted;
+}
+
+// Enqueues nsteps of the resident loop.  The remainders start from lo_in
+// (nullptr: zero) and end in d_lo.
+void enqueue_loop(fv_mesh* m, void* U, int64_t nsteps, double cfl, double t_stop, int32_t scheme,
+                  const uint2* lo_in, cudaStream_t s) {
+  fv::LoopArgs a{};
+  a.U = static_cast<float4*>(U);
+  a.lo_in = lo_in;
+  a.lo_out = m->d_lo;
+  a.geom = m->loop_geom;
+  a.ln = m->loop_ln;
+  a.ord = m->loop_ord;
+  a.info = m->loop_info;
+  a.ring_id = m->loop_ring;
+  a.push = m->loop_push;
+  a.cap = m->loop_cap;
+  a.n = (int)m->h.n;
+  a.tile = m->loop_tile;
+  a.n_tiles = m->loop_tiles;
+  double ui[4];
+  m->uinf_conserved(ui);
+  for (int q = 0; q < 4; ++q) a.uinf[q] = (float)ui[q];
+  a.cfl = cfl;
+  a.t_stop = t_stop;
+  a.fixed_dt = !(cfl > 0.0);
+  a.clamp = t_stop > 0.0;
+  a.polls = kLoopPolls;
+  a.steps_per_bound = m->blocking;
+  a.t = &m->d_scal->t[0];
+  a.err = &m->d_scal->err;
+  FV_CUDA(fv::launch_init_scalars(m->d_scal, s));
+  for (int64_t done = 0; done < nsteps; done += a.nsteps) {
+    a.nsteps = (int)std::min(nsteps - done, kLoopSteps);
+    FV_CUDA(fv::launch_loop(a, scheme == FV_SCHEME_RK2, m->use_lo(),
+                            m->wave == FV_WAVE_MAX ? fv::kWaveMax : fv::kWaveAverage, s));
+    a.lo_in = m->d_lo;  // the next launch goes on from there
+  }
+}
+
 void capture_graph(fv_mesh* m, void* U, double cfl, double t_stop, int32_t scheme,
                    const fv_closure* cl) {
   m->drop_graph();
@@ -784,6 +914,7 @@ int fv_mesh_set_variant(fv_mesh* mesh, int32_t variant) {
     if (variant == fv::kFaceTileVariant && mesh->vertex_tiles())
       invalid("normals from node coordinates run the tile shape 6");
     mesh->variant = variant;
+    mesh->loop_wanted = false;
     mesh->drop_graph();
   });
 }
@@ -794,6 +925,7 @@ int fv_mesh_set_blocking(fv_mesh* mesh, int32_t steps_per_launch, int32_t tile_c
     check_mesh(mesh);
     if (steps_per_launch != 1 && steps_per_launch != 2) invalid("steps_per_launch must be 1 or 2");
     if (staged != 0 && staged != 1) invalid("staged must be 0 or 1");
+    const bool pair_default = tile_cells == 0 && !staged;
     if (tile_cells == 0) tile_cells = 1024;
     bool known = false;
     for (int t : fv::kPairTiles) known = known || t == tile_cells;
@@ -810,6 +942,7 @@ int fv_mesh_set_blocking(fv_mesh* mesh, int32_t steps_per_launch, int32_t tile_c
     mesh->blocking = steps_per_launch;
     mesh->pair_tile = tile_cells;
     mesh->pair_staged = staged;
+    mesh->pair_default = pair_default;
     mesh->drop_graph();
   });
 }
@@ -880,6 +1013,7 @@ int fv_mesh_set_geometry(fv_mesh* mesh, int32_t form) {
       }
       mesh->geometry = form;
       mesh->variant = fv::kTileVariant;
+      mesh->loop_wanted = false;
     } else {
       invalid("unknown geometry form");
     }
@@ -949,6 +1083,9 @@ int fv_mesh_autotune(fv_mesh* mesh, const void* U, int32_t scheme, void* stream,
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     double times[fv::kStepVariants];
     const int keep = mesh->variant, keep_tile = mesh->pair_tile;
+    const bool keep_loop = mesh->loop_wanted;
+    const int blocking = mesh->blocking;
+    double loop_us = INFINITY;
     int best_tile[fv::kStepVariants];
     for (int v = 0; v < fv::kStepVariants; ++v) best_tile[v] = keep_tile;
     try {
@@ -996,9 +1133,26 @@ int fv_mesh_autotune(fv_mesh* mesh, const void* U, int32_t scheme, void* stream,
           }
         }
       }
+      // the resident loop against them, over the same steps
+      mesh->blocking = 1;
+      mesh->loop_wanted = true;
+      if (uses_loop(mesh, nullptr)) {
+        FV_CUDA(cudaMemcpyAsync(tmp, U, n * mesh->rec_bytes(), cudaMemcpyDeviceToDevice, s));
+        enqueue_loop(mesh, tmp, 2, cfl, 0.0, scheme, nullptr, s);
+        FV_CUDA(cudaEventRecord(e0, s));
+        enqueue_loop(mesh, tmp, steps, cfl, 0.0, scheme, nullptr, s);
+        FV_CUDA(cudaEventRecord(e1, s));
+        FV_CUDA(cudaEventSynchronize(e1));
+        float ms = 0.f;
+        FV_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+        loop_us = 1e3 * ms / (double)steps;
+      }
+      mesh->blocking = blocking;
     } catch (...) {
       mesh->variant = keep;
       mesh->pair_tile = keep_tile;
+      mesh->loop_wanted = keep_loop;
+      mesh->blocking = blocking;
       if (e0) cudaEventDestroy(e0);
       if (e1) cudaEventDestroy(e1);
       cudaFree(tmp);
@@ -1012,6 +1166,7 @@ int fv_mesh_autotune(fv_mesh* mesh, const void* U, int32_t scheme, void* stream,
     for (int v = 0; v < fv::kStepVariants; ++v)
       if (times[v] < times[b]) b = v;
     mesh->variant = b;
+    mesh->loop_wanted = loop_us < times[b];
     // the tile size of the tiled shapes: the fastest for shape 6 when it wins
     // (two steps per launch keep their own tile size: the two-step kernel
     // takes the standard sizes only)
@@ -1062,6 +1217,7 @@ int fv_mesh_debug_set_index(fv_mesh* mesh, int32_t table, int64_t cell, int32_t 
     if (cell < 0 || cell >= mesh->h.n || slot < 0 || slot > 2) invalid("cell or slot out of range");
     cudaStream_t s = as_stream(stream);
     ensure_device(mesh, s);
+    mesh->loop_wanted = false;  // the loop has tables of its own
     if (table == 0) {
       // global neighbour ids: FP32 keeps face 0's in the geometry record
       if (mesh->f64()) {
@@ -1109,9 +1265,22 @@ int fv_step(fv_mesh* mesh, void* U, int64_t nsteps, double cfl, double t_stop, i
     ensure_device(mesh, s);
     if (closure) ensure_faces(mesh, s);
     const int64_t n = mesh->h.n;
-    FV_CUDA(fv::launch_init_scalars(mesh->d_scal, s));
     mesh->last_t_slot = 0;
     mesh->stepped = true;
+    if (n > 0 && nsteps > 0 && uses_loop(mesh, closure)) {
+      if (mesh->blocking == 2) check_tile_smem(mesh, pair_smem(mesh));
+      const bool keep = mesh->use_lo() && mesh->user_lo;
+      if (keep)  // the remainder the caller kept from the last call
+        FV_CUDA(cudaMemcpyAsync(mesh->d_lo, mesh->user_lo, n * sizeof(uint2),
+                                cudaMemcpyDeviceToDevice, s));
+      enqueue_loop(mesh, U, nsteps, cfl, t_stop, scheme, keep ? mesh->d_lo : nullptr, s);
+      if (keep)
+        FV_CUDA(cudaMemcpyAsync(mesh->user_lo, mesh->d_lo, n * sizeof(uint2),
+                                cudaMemcpyDeviceToDevice, s));
+      if (t_advanced) read_status(mesh, s, t_advanced, true);
+      return;
+    }
+    FV_CUDA(fv::launch_init_scalars(mesh->d_scal, s));
     if (n > 0 && nsteps > 0) {
       if (mesh->use_lo()) {
         if (mesh->user_lo)  // the remainder the caller kept from the last call

@@ -386,22 +386,15 @@ __device__ __forceinline__ R geom_inradius(const rec_t<R>* __restrict__ geom, in
   return inradius<R>(g1, perim);
 }
 
-// Everything after the face fluxes: residual output, or the forward-Euler /
-// Heun update (plain or compensated) and the CFL bound of the new state.
-// acc holds twice the flux sum (face_flux_acc): the factors applied to it
-// carry the 1/2 (exactly).
+// The new state of one cell from twice its flux sum (face_flux_acc): the
+// forward-Euler or Heun update, plain or compensated.  The factors applied to
+// acc carry the 1/2 (exactly).  COMP: lo is the remainder of U^n (of the
+// stage's start), lo_stage that of U* (second Heun stage); lo_out receives the
+// remainder of the new state.  base: U^n (second Heun stage).
 template <typename R, int MODE, bool COMP>
-__device__ __forceinline__ void finish_cell(const StepArgs& a, rec_t<R>* out, int64_t i,
-                                            const CellIn<R>& c, const R acc[4], R perim, R dt,
-                                            R& bmin, bool& ok) {
-  const rec_t<R>& UL = c.U;
-  const R invV = c.g1.z;
-  bool cell_ok = true;
-  if (MODE == kModeResidual) {
-    const R m = mul(R(-0.5), invV);
-    out[i] = Rec<R>::make(mul(m, acc[0]), mul(m, acc[1]), mul(m, acc[2]), mul(m, acc[3]));
-    return;
-  }
+__device__ __forceinline__ rec_t<R> advance_state(const rec_t<R>& UL, const rec_t<R>& base_rec,
+                                                  const R acc[4], R invV, R dt, uint2 lo_in,
+                                                  uint2 lo_stage, uint2& lo_out) {
   if (COMP) {
     // float state + bfloat16 remainder: the increment and the remainder are
     // added with an exact TwoSum, and what the float sum drops becomes the
@@ -411,18 +404,14 @@ __device__ __forceinline__ void finish_cell(const StepArgs& a, rec_t<R>* out, in
     float base[4] = {u[0], u[1], u[2], u[3]};
     float inc[4];
     float lo[4];
-    if (MODE == kModeRK2b) {
-      base[0] = (float)c.base.x, base[1] = (float)c.base.y, base[2] = (float)c.base.z,
-      base[3] = (float)c.base.w;
-    }
-    unpack_rem(c.lo, lo);  // the remainder of U^n
+    unpack_rem(lo_in, lo);  // the remainder of U^n
     if (MODE == kModeRK2b) {
       // U^{n+1} = U^n + (U* - U^n)/2 + dt R(U*)/2, with U^n = base + lo and
       // U* = u + lo_stage
-      base[0] = (float)c.base.x, base[1] = (float)c.base.y, base[2] = (float)c.base.z,
-      base[3] = (float)c.base.w;
+      base[0] = (float)base_rec.x, base[1] = (float)base_rec.y, base[2] = (float)base_rec.z,
+      base[3] = (float)base_rec.w;
       float ls[4];
-      unpack_rem(c.lo_stage, ls);
+      unpack_rem(lo_stage, ls);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         inc[q] = fma_(0.5f, sub(u[q], base[q]),
@@ -434,28 +423,45 @@ __device__ __forceinline__ void finish_cell(const StepArgs& a, rec_t<R>* out, in
     float sm[4], e[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) sm[q] = two_sum(base[q], inc[q], e[q]);
-    const rec_t<R> Un = Rec<R>::make(R(sm[0]), R(sm[1]), R(sm[2]), R(sm[3]));
-    out[i] = Un;
-    if (MODE == kModeRK2a) {
-      a.lo_stage[i] = pack_rem(e);
-    } else {
-      a.lo[i] = pack_rem(e);
-      bmin = fmin(bmin, cell_bound<R>(Un, inradius<R>(c.g1, perim), cell_ok));
-    }
-  } else {
-    const R f = mul(mul(R(-0.5), dt), invV);
-    rec_t<R> Un = Rec<R>::make(fma_(f, acc[0], UL.x), fma_(f, acc[1], UL.y),
-                               fma_(f, acc[2], UL.z), fma_(f, acc[3], UL.w));
-    if (MODE == kModeRK2b) {
-      const rec_t<R>& B = c.base;
-      const R h = R(0.5);
-      Un = Rec<R>::make(add(mul(h, B.x), mul(h, Un.x)), add(mul(h, B.y), mul(h, Un.y)),
-                        add(mul(h, B.z), mul(h, Un.z)), add(mul(h, B.w), mul(h, Un.w)));
-    }
-    out[i] = Un;
-    if (MODE != kModeRK2a) bmin = fmin(bmin, cell_bound<R>(Un, inradius<R>(c.g1, perim), cell_ok));
+    lo_out = pack_rem(e);
+    return Rec<R>::make(R(sm[0]), R(sm[1]), R(sm[2]), R(sm[3]));
   }
-  ok = ok && cell_ok;
+  const R f = mul(mul(R(-0.5), dt), invV);
+  rec_t<R> Un = Rec<R>::make(fma_(f, acc[0], UL.x), fma_(f, acc[1], UL.y), fma_(f, acc[2], UL.z),
+                             fma_(f, acc[3], UL.w));
+  if (MODE == kModeRK2b) {
+    const rec_t<R>& B = base_rec;
+    const R h = R(0.5);
+    Un = Rec<R>::make(add(mul(h, B.x), mul(h, Un.x)), add(mul(h, B.y), mul(h, Un.y)),
+                      add(mul(h, B.z), mul(h, Un.z)), add(mul(h, B.w), mul(h, Un.w)));
+  }
+  return Un;
+}
+
+// Everything after the face fluxes: residual output, or the update
+// (advance_state) and the CFL bound of the new state.
+template <typename R, int MODE, bool COMP>
+__device__ __forceinline__ void finish_cell(const StepArgs& a, rec_t<R>* out, int64_t i,
+                                            const CellIn<R>& c, const R acc[4], R perim, R dt,
+                                            R& bmin, bool& ok) {
+  const R invV = c.g1.z;
+  if (MODE == kModeResidual) {
+    const R m = mul(R(-0.5), invV);
+    out[i] = Rec<R>::make(mul(m, acc[0]), mul(m, acc[1]), mul(m, acc[2]), mul(m, acc[3]));
+    return;
+  }
+  uint2 lo_out;
+  const rec_t<R> Un =
+      advance_state<R, MODE, COMP>(c.U, c.base, acc, invV, dt, c.lo, c.lo_stage, lo_out);
+  out[i] = Un;
+  if (MODE == kModeRK2a) {
+    if (COMP) a.lo_stage[i] = lo_out;
+  } else {
+    if (COMP) a.lo[i] = lo_out;
+    bool cell_ok;
+    bmin = fmin(bmin, cell_bound<R>(Un, inradius<R>(c.g1, perim), cell_ok));
+    ok = ok && cell_ok;
+  }
 }
 
 }  // namespace

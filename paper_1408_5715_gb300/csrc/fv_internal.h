@@ -105,6 +105,26 @@ struct PairTiles {
 };
 PairTiles build_pair_tiles(const HostMesh& m, int32_t tile);
 
+// Tiles of the resident loop (loop_step.cu): block b keeps the cells
+// [b*tile, min((b+1)*tile, n)) on chip for a whole time loop.  Inside a tile
+// the cells are numbered with those that border another tile first (its edge
+// cells), then the rest, each part in ascending id; the tile's ring (cells of
+// other tiles adjacent to it, ascending id) is numbered from `tile` on.
+struct LoopTiles {
+  int32_t tile = 0;
+  int32_t n_tiles = 0;
+  int32_t cap = 0;                // tile + the largest ring
+  std::vector<int32_t> info;      // [4 n_tiles] ring offset, ring size, edge cells, first edge cell
+  std::vector<int32_t> ord;       // [n] global id of the cell at position b*tile + e
+  std::vector<uint32_t> cell_ln;  // [2 n] by position: tile-local neighbours (as PairTiles)
+  std::vector<int32_t> ring_id;   // the rings' cells
+  // [3 edge cells of all tiles] per face: tile << 16 | entry of the ring of
+  // the tile across that the cell is, or all ones (no other tile across, or
+  // the tile of a lower face)
+  std::vector<uint32_t> push;
+};
+LoopTiles build_loop_tiles(const HostMesh& m, int32_t tile);
+
 // The nodes of each tile for normals formed from vertex coordinates
 // (vertex_geom.cpp).  Tile b's nodes are vq[2 voff[b] ..] (grid coordinates,
 // duplicated where tiles share nodes); each cell's three nodes are 16-bit

@@ -247,6 +247,41 @@ inline size_t pair_smem_bytes(int e_cap, int t1_cap, int tile, bool staged) {
 // arrive by bulk copies (cp.async.bulk) into double-buffered stages
 cudaError_t launch_step_pair(const PairArgs& a, int staged, cudaStream_t s);
 
+// A whole time loop in one launch of one thread-block cluster, every block
+// keeping its tile on chip (loop_step.cu; FP32).  Arrays in the order of
+// build_loop_tiles.
+struct LoopArgs {
+  float4* U;                  // state, advanced in place (cell order)
+  const uint2* lo_in;         // compensated update: remainders at the start (nullptr: zero) ...
+  uint2* lo_out;              // ... and at the end, in cell order
+  const float4* geom;         // 2 records per cell, loop order
+  const uint2* ln;            // tile-local neighbours, loop order
+  const int* ord;             // cell of each position
+  const int4* info;           // [kLoopMaxTiles] ring offset, ring size, edge cells, first push
+  const int* ring_id;         // the rings' cells
+  const unsigned* push;       // [3 per edge cell] tile << 16 | entry of its ring, or all ones
+  int n, tile, n_tiles, cap;  // cap: cells of a tile and the largest ring
+  float uinf[4];
+  double cfl, t_stop;         // as StepArgs; with fixed_dt (cfl < 0), clamp (t_stop > 0)
+  bool fixed_dt, clamp;
+  unsigned polls;             // tries of a wait before it gives up (error bit 2)
+  int nsteps;
+  int steps_per_bound;        // 1, or 2: two steps share one CFL bound
+  double* t;                  // time advanced, read and written
+  int* err;
+};
+constexpr int kLoopMaxTiles = 16;  // blocks of one (non-portable) cluster
+constexpr int kLoopMaxTile = 768;  // cells of a block: one per thread
+// dynamic shared memory: two states per cell, and the remainders (two with RK2)
+inline size_t loop_smem_bytes(int cap, int tile, bool comp, bool rk2) {
+  return (size_t)cap * 32 + (comp ? (size_t)tile * (rk2 ? 16 : 8) : 0);
+}
+cudaError_t launch_loop(const LoopArgs& a, bool rk2, bool comp, int wave, cudaStream_t s);
+// clusters of that launch the device can hold at a time (a.tile, a.n_tiles, a.cap)
+cudaError_t loop_clusters(const LoopArgs& a, bool rk2, bool comp, int* clusters);
+cudaError_t launch_loop_geometry(const float4* geom, const int* ord, int n, float4* out,
+                                 cudaStream_t s);
+
 // float (FV_F32) or double (FV_F64) instantiations
 cudaError_t launch_step(bool f64, int mode, int variant, const StepArgs& a, cudaStream_t s);
 cudaError_t launch_init_scalars(LoopScalars* d, cudaStream_t s);

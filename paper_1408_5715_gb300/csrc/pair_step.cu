@@ -66,25 +66,11 @@ __device__ __forceinline__ int halo_cell(const PairArgs& a, int j) {
   return index_ok(g, a.n, a.err) ? g : 0;
 }
 
-// Forward-Euler update of one cell, plain or compensated (the arithmetic of
-// the one-step kernel's update).
+// Forward-Euler update of one cell, plain or compensated.
 template <bool COMP>
 __device__ __forceinline__ float4 fe_update(const float4& UL, float invV, const float acc[4],
                                             float dt, uint2 lo_in, uint2& lo_out) {
-  // acc holds twice the flux sum (face_flux_acc)
-  if (COMP) {
-    const float f = mul(mul(-0.5f, dt), invV);
-    const float u[4] = {UL.x, UL.y, UL.z, UL.w};
-    float lo[4], s[4], e[4];
-    unpack_rem(lo_in, lo);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) s[q] = two_sum(u[q], fma_(f, acc[q], lo[q]), e[q]);
-    lo_out = pack_rem(e);
-    return make_float4(s[0], s[1], s[2], s[3]);
-  }
-  const float f = mul(mul(-0.5f, dt), invV);
-  return make_float4(fma_(f, acc[0], UL.x), fma_(f, acc[1], UL.y), fma_(f, acc[2], UL.z),
-                     fma_(f, acc[3], UL.w));
+  return advance_state<float, kModeFE, COMP>(UL, UL, acc, invV, dt, lo_in, lo_in, lo_out);
 }
 
 // dt of both steps of the pair, as the one-step kernel would take them

@@ -1,5 +1,5 @@
 // tiles.cpp -- tiles and their halos for the two-step (temporally blocked)
-// update.
+// update, and the tiles of the resident loop (build_loop_tiles).
 //
 // Chaining two updates of a cell without going back to memory (the paper's
 // processor chaining, Sec. 7) needs, for a set of cells, the states of
@@ -134,6 +134,83 @@ PairTiles build_pair_tiles(const HostMesh& m, int32_t tile) {
   L.tile_info[2 * L.n_tiles] = (int32_t)L.halo_id.size();
   L.face_off.push_back((int32_t)(L.face_rec.size() / 2));
   if (L.face_rec.size() / 2 > (size_t)INT32_MAX) throw Error{FV_EINVAL, "too many tile faces"};
+  return L;
+}
+
+LoopTiles build_loop_tiles(const HostMesh& m, int32_t tile) {
+  const int64_t n = m.n;
+  if (tile < 1 || n > INT32_MAX || (n + tile - 1) / tile >= 0xFFFF)
+    throw Error{FV_EINVAL, "resident loop: bad tile size"};
+  LoopTiles L;
+  L.tile = L.cap = tile;
+  L.n_tiles = (int32_t)((n + tile - 1) / tile);
+  L.info.assign(4 * (size_t)L.n_tiles, 0);
+  L.ord.resize((size_t)n);
+  L.cell_ln.resize(2 * (size_t)n);
+  std::vector<int32_t> pos((size_t)n);  // local position of every cell in its tile
+  std::vector<int32_t> inner, ring;
+  int32_t edge_cells = 0;
+  for (int32_t b = 0; b < L.n_tiles; ++b) {
+    const int32_t t0 = b * tile, t1 = (int32_t)std::min<int64_t>((int64_t)t0 + tile, n);
+    auto outside = [&](int32_t x) { return x >= 0 && (x < t0 || x >= t1); };
+    inner.clear();
+    ring.clear();
+    int32_t at = t0;
+    for (int32_t c = t0; c < t1; ++c) {
+      const int32_t* x = &m.nbr[3 * (size_t)c];
+      if (!outside(x[0]) && !outside(x[1]) && !outside(x[2])) {
+        inner.push_back(c);
+        continue;
+      }
+      pos[c] = at - t0;
+      L.ord[at++] = c;
+      for (int k = 0; k < 3; ++k)
+        if (outside(x[k])) ring.push_back(x[k]);
+    }
+    const int32_t edges = at - t0;
+    for (int32_t c : inner) {
+      pos[c] = at - t0;
+      L.ord[at++] = c;
+    }
+    std::sort(ring.begin(), ring.end());
+    ring.erase(std::unique(ring.begin(), ring.end()), ring.end());
+    if (tile + (int64_t)ring.size() > kLocalLimit)
+      throw Error{FV_EINVAL, "resident loop: a tile with its ring exceeds 65533 cells"};
+    L.cap = std::max(L.cap, tile + (int32_t)ring.size());
+    L.info[4 * b] = (int32_t)L.ring_id.size();
+    L.info[4 * b + 1] = (int32_t)ring.size();
+    L.info[4 * b + 2] = edges;
+    L.info[4 * b + 3] = edge_cells;
+    edge_cells += edges;
+    L.ring_id.insert(L.ring_id.end(), ring.begin(), ring.end());
+  }
+  // the entry of cell c in tile b's ring
+  auto entry = [&](int32_t b, int32_t c) {
+    const auto r0 = L.ring_id.begin() + L.info[4 * b], r1 = r0 + L.info[4 * b + 1];
+    return (uint32_t)(std::lower_bound(r0, r1, c) - r0);
+  };
+  L.push.assign(3 * (size_t)edge_cells, 0xFFFFFFFFu);
+  for (int32_t p = 0; p < (int32_t)n; ++p) {
+    const int32_t b = p / tile, t0 = b * tile, e = p - t0, c = L.ord[p];
+    const int32_t* x = &m.nbr[3 * (size_t)c];
+    uint32_t v[3];
+    for (int k = 0; k < 3; ++k) {
+      const int32_t bx = x[k] < 0 ? b : x[k] / tile;
+      if (x[k] < 0) {
+        v[k] = (uint32_t)(0x10000 + x[k]);
+      } else if (bx == b) {
+        v[k] = (uint32_t)pos[x[k]];
+      } else {
+        v[k] = (uint32_t)tile + entry(b, x[k]);
+        bool sent = false;
+        for (int q = 0; q < k; ++q) sent = sent || (x[q] >= 0 && x[q] / tile == bx);
+        if (!sent)
+          L.push[3 * (size_t)(L.info[4 * b + 3] + e) + k] = (uint32_t)bx << 16 | entry(bx, c);
+      }
+    }
+    L.cell_ln[2 * (size_t)p] = v[0] | (v[1] << 16);
+    L.cell_ln[2 * (size_t)p + 1] = v[2];
+  }
   return L;
 }
 
