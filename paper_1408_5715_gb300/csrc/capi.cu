@@ -95,12 +95,11 @@ struct fv_closure {
   // graph captured with other parameters (b3 is baked into its launches) or
   // with another closure at the same address is recaptured
   uint64_t version = 0;
-  // training scratch: per-block gradient and loss partials, outputs
-  int grad_blocks = 0;
-  float* d_gpart = nullptr;
-  double* d_lpart = nullptr;
+  // training scratch: per-cell terms, per-block gradient and loss partials
+  // (scratch.cells grows to the largest mesh trained on)
+  fv::ClosureScratch scratch{};
+  int64_t cells_cap = 0;
   float* d_grad = nullptr;
-  double* d_loss = nullptr;
 
   fv::ClosureParams params() const {
     fv::ClosureParams p;
@@ -1987,22 +1986,24 @@ int fv_closure_create(const float* theta, fv_closure** out) {
       FV_CUDA(cudaMalloc((void**)&c->d_w2, 32 * 16 * sizeof(unsigned)));
       FV_CUDA(cudaMalloc((void**)&c->d_b, 97 * sizeof(float)));
       FV_CUDA(cudaMalloc((void**)&c->d_theta, fv::kClosureParams * sizeof(float)));
-      c->grad_blocks = fv::closure_grad_blocks();
-      FV_CUDA(cudaMalloc((void**)&c->d_gpart,
-                         (size_t)c->grad_blocks * fv::kClosureParams * sizeof(float)));
-      FV_CUDA(cudaMalloc((void**)&c->d_lpart, (size_t)c->grad_blocks * sizeof(double)));
+      fv::ClosureScratch& t = c->scratch;
+      t.grad_blocks = fv::closure_grad_blocks();
+      t.loss_blocks = fv::closure_loss_blocks();
+      FV_CUDA(cudaMalloc((void**)&t.gpart,
+                         (size_t)t.grad_blocks * fv::kClosureParams * sizeof(float)));
+      FV_CUDA(cudaMalloc((void**)&t.lpart, (size_t)t.loss_blocks * sizeof(double)));
       FV_CUDA(cudaMalloc((void**)&c->d_grad, fv::kClosureParams * sizeof(float)));
-      FV_CUDA(cudaMalloc((void**)&c->d_loss, sizeof(double)));
+      FV_CUDA(cudaMalloc((void**)&t.loss, sizeof(double)));
       closure_upload(c, theta, false, nullptr);
     } catch (...) {
       cudaFree(c->d_w1);
       cudaFree(c->d_w2);
       cudaFree(c->d_b);
       cudaFree(c->d_theta);
-      cudaFree(c->d_gpart);
-      cudaFree(c->d_lpart);
+      cudaFree(c->scratch.gpart);
+      cudaFree(c->scratch.lpart);
       cudaFree(c->d_grad);
-      cudaFree(c->d_loss);
+      cudaFree(c->scratch.loss);
       delete c;
       throw;
     }
@@ -2018,10 +2019,11 @@ int fv_closure_destroy(fv_closure* closure) {
     cudaFree(closure->d_w2);
     cudaFree(closure->d_b);
     cudaFree(closure->d_theta);
-    cudaFree(closure->d_gpart);
-    cudaFree(closure->d_lpart);
+    cudaFree(closure->scratch.cells);
+    cudaFree(closure->scratch.gpart);
+    cudaFree(closure->scratch.lpart);
     cudaFree(closure->d_grad);
-    cudaFree(closure->d_loss);
+    cudaFree(closure->scratch.loss);
     delete closure;
   });
 }
@@ -2079,14 +2081,18 @@ int fv_closure_loss_grad(fv_mesh* mesh, const void* U0, const void* Ut, double d
     ensure_device(mesh, s);
     fv::StepArgs a = base_args(mesh);
     a.U = U0;
+    if (closure->cells_cap < mesh->h.n) {
+      // the stream may still read the smaller array (cudaFree waits for it)
+      dev_free(closure->scratch.cells);
+      closure->cells_cap = 0;
+      FV_CUDA(cudaMalloc((void**)&closure->scratch.cells, mesh->h.n * sizeof(float4)));
+      closure->cells_cap = mesh->h.n;
+    }
     FV_CUDA(fv::launch_closure_grad(a, static_cast<const float*>(Ut), dt, weights,
-                                    closure->params(), closure->d_gpart, closure->d_lpart,
-                                    closure->grad_blocks, closure->d_grad, closure->d_loss, s));
-    if (grad)
-      FV_CUDA(cudaMemcpyAsync(grad, closure->d_grad, fv::kClosureParams * sizeof(float),
-                              cudaMemcpyDeviceToDevice, s));
+                                    closure->params(), closure->scratch,
+                                    grad ? grad : closure->d_grad, s));
     if (loss) {
-      FV_CUDA(cudaMemcpyAsync(loss, closure->d_loss, sizeof(double), cudaMemcpyDeviceToHost, s));
+      FV_CUDA(cudaMemcpyAsync(loss, closure->scratch.loss, sizeof(double), cudaMemcpyDeviceToHost, s));
       FV_CUDA(cudaStreamSynchronize(s));
     }
   });

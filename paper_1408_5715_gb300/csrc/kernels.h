@@ -159,13 +159,21 @@ cudaError_t launch_step_scaled(int mode, const StepArgs& a, const float* s_cf, c
 size_t closure_tile_smem_bytes(int t1_cap, int tile, bool tc);
 cudaError_t launch_step_closure_tile(int mode, const StepArgs& a, const ClosureParams& cp,
                                      cudaStream_t s);
-// Blocks the gradient kernel launches at most on this device.
+// Blocks the two training kernels launch at most on this device.
 int closure_grad_blocks();
-// One-step loss and gradient; gpart [max_blocks * kClosureParams], lpart
-// [max_blocks] scratch; grad [kClosureParams] and loss [1] device outputs.
+int closure_loss_blocks();
+// Device scratch of the training kernels.
+struct ClosureScratch {
+  float4* cells;  // [n] per cell: dL/dU1 (-dt/V)
+  float* gpart;   // [grad_blocks * kClosureParams]
+  double* lpart;  // [loss_blocks]
+  double* loss;   // [1], written
+  int grad_blocks, loss_blocks;
+};
+// One-step loss and gradient (grad: [kClosureParams], written).
 cudaError_t launch_closure_grad(const StepArgs& a, const float* Ut, double dt, const double* w,
-                                const ClosureParams& cp, float* gpart, double* lpart,
-                                int max_blocks, float* grad, double* loss, cudaStream_t s);
+                                const ClosureParams& cp, const ClosureScratch& sc, float* grad,
+                                cudaStream_t s);
 cudaError_t launch_adam(float* theta, const float* grad, float* m, float* v, int n, double lr,
                         double b1, double b2, double eps, int64_t step, cudaStream_t s);
 // theta (device, FP32, kClosureParams) -> w1, w2 (bfloat16 pairs), b (b1 b2 w3 b3)
