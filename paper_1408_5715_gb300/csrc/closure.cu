@@ -963,7 +963,8 @@ unsigned cl_grid(K kernel, int64_t items_per_warp_group, int64_t n) {
 // bias made the gradient's error 2.4e-7, against 1.8e-7 for FP32 sums).
 // Measured on 250,000 cells: 275 us for the former row-by-row backward (lane o
 // a unit, 64 shuffles and shared-memory reads per row, every face from both
-// sides) against CELLS us + GRAD us.
+// sides) against 27 + 44 us (ncu); a training iteration (loss, gradient, Adam,
+// new weights) 460 -> 150 us.
 // ---------------------------------------------------------------------------
 constexpr int kGrWarps = 4;
 constexpr int kGrThreads = 32 * kGrWarps;
