@@ -266,16 +266,34 @@ bool tiled_shape(int v) { return v == fv::kTileVariant || v == fv::kFaceTileVari
 bool uses_tiles(const fv_mesh* m) { return m->blocking == 2 || tiled_shape(m->variant); }
 
 // The faces each tile evaluates once (shape 7), uploaded when that shape
-// first runs on the current tiles.
+// first runs on the current tiles: FP32 two words per face (tiles.cpp), FP64
+// the face's normal, its length (as the kernels form it: correctly rounded)
+// and the two words, 32 bytes.
 void upload_tile_faces(fv_mesh* m, const fv::PairTiles& L, cudaStream_t s) {
+  const size_t nf = L.face_rec.size() / 2;
+  std::vector<double> rec;
+  if (m->f64()) {
+    rec.resize(4 * nf);
+    for (size_t b = 0; b + 1 < L.face_off.size(); ++b)
+      for (int32_t f = L.face_off[b]; f < L.face_off[b + 1]; ++f) {
+        const uint32_t* w = &L.face_rec[2 * (size_t)f];
+        const double* n = &m->h.nrm[2 * (3 * (b * (size_t)L.tile + (w[0] & 0xFFFFu)) +
+                                         ((w[0] >> 16) & 3u))];
+        double* r = &rec[4 * (size_t)f];
+        r[0] = n[0];
+        r[1] = n[1];
+        r[2] = std::sqrt(std::fma(n[0], n[0], n[1] * n[1]));
+        std::memcpy(r + 3, w, 2 * sizeof(uint32_t));
+      }
+  }
+  const void* src = m->f64() ? static_cast<const void*>(rec.data()) : L.face_rec.data();
+  const size_t bytes = nf * (m->f64() ? 32 : 8);
   FV_CUDA(cudaMalloc((void**)&m->d_face_off, L.face_off.size() * sizeof(int32_t)));
-  FV_CUDA(cudaMalloc((void**)&m->d_face_rec, std::max<size_t>(L.face_rec.size(), 2) *
-                                                  sizeof(uint32_t)));
+  FV_CUDA(cudaMalloc((void**)&m->d_face_rec, std::max<size_t>(bytes, 8)));
   FV_CUDA(cudaMemcpyAsync(m->d_face_off, L.face_off.data(), L.face_off.size() * sizeof(int32_t),
                           cudaMemcpyHostToDevice, s));
-  FV_CUDA(cudaMemcpyAsync(m->d_face_rec, L.face_rec.data(), L.face_rec.size() * sizeof(uint32_t),
-                          cudaMemcpyHostToDevice, s));
-  FV_CUDA(cudaStreamSynchronize(s));  // L is a staging buffer
+  if (bytes) FV_CUDA(cudaMemcpyAsync(m->d_face_rec, src, bytes, cudaMemcpyHostToDevice, s));
+  FV_CUDA(cudaStreamSynchronize(s));  // L and rec are staging buffers
 }
 
 void ensure_tiles(fv_mesh* m, cudaStream_t s) {
@@ -371,7 +389,7 @@ std::vector<int> tile_candidates(int64_t n) {
   int dev = 0, sms = 0;
   FV_CUDA(cudaGetDevice(&dev));
   FV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  for (int b : {5, 4, 2})  // resident blocks per SM of the FP32 / FP64 shapes
+  for (int b : {5, 4, 3, 2})  // resident blocks per SM of the FP32 / FP64 shapes
     for (int w = 1; w <= 3; ++w) {
       const int64_t slots = (int64_t)w * b * sms;
       const int64_t c = ((n + slots - 1) / slots + 31) / 32 * 32;

@@ -49,34 +49,70 @@ struct Rec<double> {
 template <typename R>
 using rec_t = typename Rec<R>::T;
 
-// Reciprocal and square root.  FP64 keeps the correctly rounded operations
-// (its results are held to 1e-12 of the FP64 oracle).  The FP32 path is
-// memory-bound and its error budget is set by float rounding, so it uses the
-// single-instruction approximations of the special-function unit
-// (relative error about 2^-23).
+// Reciprocal and square root.  The FP32 path is memory-bound and its error
+// budget is set by float rounding, so it uses the single-instruction
+// approximations of the special-function unit (relative error about 2^-23).
+//
+// FP64 is bound by GB300's FP64 pipe (two lanes a clock and SM, a sixty-fourth
+// of the FP32 rate), so its forms spend as few FP64 operations as they can: the
+// special-function unit's FP32 result is the start value y0 (24 bits, relative
+// error below 2^-21; the conversions are integer shifts), and
+//   1/x:      one step of third order, y0 (1 + e + e^2) with e = 1 - x y0 exact
+//             to 2^-53 e: three operations, the remainder e^3 below 2^-63;
+//   sqrt(a):  a Newton step on g = a y0, then Markstein's last step (IBM J.
+//             Res. Dev. 34(1), 1990): g + (a - g^2) y0/2 with the residual
+//             a - g^2 exact in an FMA: five operations.
+// Both round almost always as the exact value does (error at most 0.5 ulp plus
+// a few 2^-10; compared with the correctly rounded operations in
+// test_gpu_fp64_faces.py).  Arguments outside [2^-100, 2^100) -- zero, negative
+// and non-finite ones among them -- take the correctly rounded operations.
 template <typename R>
 __device__ __forceinline__ R recip(R x);
-template <>
-__device__ __forceinline__ double recip<double>(double x) {
-  return 1.0 / x;
+template <typename R>
+__device__ __forceinline__ R root(R x);
+
+__device__ __forceinline__ bool in_quick_range(double x) {
+  return (unsigned)__double2hiint(x) - (923u << 20) < (200u << 20);
 }
+// x rounded toward zero to float, and a positive normal float widened, for
+// values in the quick range.
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned w = __funnelshift_l((unsigned)__double2loint(x), (unsigned)__double2hiint(x), 3);
+  return __uint_as_float((w ^ 0x40000000u) & 0x7fffffffu);
+}
+__device__ __forceinline__ double widen(float y) {
+  const unsigned b = __float_as_uint(y);
+  return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+}
+
 template <>
 __device__ __forceinline__ float recip<float>(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-template <typename R>
-__device__ __forceinline__ R root(R x);
 template <>
-__device__ __forceinline__ double root<double>(double x) {
-  return sqrt(x);
+__device__ __forceinline__ double recip<double>(double x) {
+  if (!in_quick_range(x)) return 1.0 / x;
+  const double y = widen(recip<float>(narrow(x)));
+  const double e = __fma_rn(-x, y, 1.0);
+  return __fma_rn(__fma_rn(e, e, e), y, y);
 }
 template <>
 __device__ __forceinline__ float root<float>(float x) {
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
+}
+template <>
+__device__ __forceinline__ double root<double>(double a) {
+  if (!in_quick_range(a)) return sqrt(a);
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(narrow(a)));
+  const double y = widen(r), h = widen(0.5f * r);
+  double g = __dmul_rn(a, y);
+  g = __fma_rn(g, __fma_rn(-g, h, 0.5), g);
+  return __fma_rn(__fma_rn(-g, g, a), h, g);
 }
 
 // Explicitly rounded arithmetic.  Every multiply-add of the cell update is
@@ -217,6 +253,14 @@ __device__ __forceinline__ void face_flux_value(const rec_t<R>& UL, const Prim<R
     na = -fmax(fma_(len, L.c, fabs(qL)), fma_(len, W.c, fabs(qR)));
   if (SCALED) na = mul(s, na);
   X[0] = fma_(na, sub(UR.x, UL.x), add(mul(UL.x, qL), mul(UR.x, qR)));
+  if constexpr (sizeof(R) == 8) {
+    // the sum of the two pressures once: one FP64 operation fewer
+    const R ps = add(L.p, W.p);
+    X[1] = fma_(na, sub(UR.y, UL.y), fma_(ps, nx, add(mul(UL.y, qL), mul(UR.y, qR))));
+    X[2] = fma_(na, sub(UR.z, UL.z), fma_(ps, ny, add(mul(UL.z, qL), mul(UR.z, qR))));
+    X[3] = fma_(na, sub(UR.w, UL.w), add(mul(add(UL.w, L.p), qL), mul(add(UR.w, W.p), qR)));
+    return;
+  }
   X[1] = fma_(na, sub(UR.y, UL.y),
               add(fma_(UL.y, qL, mul(L.p, nx)), fma_(UR.y, qR, mul(W.p, nx))));
   X[2] = fma_(na, sub(UR.z, UL.z),

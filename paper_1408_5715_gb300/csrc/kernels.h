@@ -80,7 +80,8 @@ struct StepArgs {
   const int* halo_id;
   int tile;
   int t1_cap;
-  // shape 7: each tile's faces evaluated once (tiles.cpp face_off / face_rec)
+  // shape 7: each tile's faces evaluated once (tiles.cpp face_off / face_rec;
+  // FP64: 32-byte records nx, ny, length and the face's two words)
   const int* tile_face_off;
   const uint2* tile_face;
   // Vertex geometry of the tile variant (FP32; vertex_geom.cpp), or nullptr:

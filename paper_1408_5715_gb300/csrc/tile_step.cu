@@ -123,11 +123,12 @@ __global__ void __launch_bounds__(THREADS, sizeof(R) == 4 ? 1280 / THREADS : 1)
 // fluxes are exactly antisymmetric (face_flux_value), so every slot holds the
 // bits the cell would compute itself.  Phase 2: every tile cell adds its three
 // slots in face order and finishes as the other shapes do: the same bits, with
-// about half the face arithmetic.  It pays where the arithmetic is the
-// bottleneck (FP64 on GB300); sF costs 3 records per tile cell of shared
-// memory.
+// about half the face arithmetic.  sF costs 3 records per tile cell of shared
+// memory.  It pays where the arithmetic is the bottleneck, in FP64, which has a
+// kernel of its own (k_step_faces64); this one is FP32's.
 template <typename R, int MODE, bool COMP, int THREADS, int KMAX, int WAVE>
 __global__ void __launch_bounds__(THREADS, 1) k_step_tile_faces(StepArgs a) {
+  static_assert(sizeof(R) == 4);
   chain_entry();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   rec_t<R>* sU = reinterpret_cast<rec_t<R>*>(smem_raw);  // [t1_cap] states
@@ -222,6 +223,153 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_tile_faces(StepArgs a) {
         *a.bmin_reset = kInfBits;
       }
     }
+  }
+}
+
+// -x without the FP64 pipe.
+__device__ __forceinline__ double flip(double x) {
+  return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x));
+}
+
+// A CFL bound in FP32 that rules most cells out of the FP64 minimum: within
+// kBoundSlack of the exact bound of a cell whose state is plainly good (true),
+// else the cell has to be evaluated exactly.
+constexpr float kBoundSlack = 5e-5f;
+
+__device__ __forceinline__ bool rough_bound(const dq4& U, double inradius, float& b) {
+  const float rho = (float)U.x, mx = (float)U.y, my = (float)U.z, E = (float)U.w,
+              r = (float)inradius;
+  const float ir = recip<float>(rho), u = mx * ir, v = my * ir;
+  const float pe = E - 0.5f * (mx * u + my * v);  // p / (gamma - 1)
+  b = r * recip<float>(root<float>(u * u + v * v) +
+                       root<float>((float)(kGamma * kGammaM1) * pe * ir));
+  // rounding moves pe by at most a few 2^-24 E: at pe > E / 100 the sound
+  // speed is good to 2e-5, and the exact pressure is positive too
+  return rho > 1e-20f && rho < 1e20f && E < 1e20f && pe > 0.01f * E && pe > 1e-20f && r > 1e-20f;
+}
+
+// Shape 7 in FP64, bound by the FP64 pipe (two lanes a clock and SM): 84 % of
+// it busy with 173 FP64 instructions per cell in the form above, of which the
+// fluxes are a third.  What is not the fluxes' is taken out:
+//   - a face's record carries its normal and length (32 bytes, read in order),
+//     so no square root per face;
+//   - the CFL bound (two square roots, two divisions) is evaluated only for
+//     cells that may be the minimum: an FP32 bound of every cell, the block's
+//     minimum of those, and FP64 for the cells within the FP32 error of it --
+//     unless the minimum so far already rules the block out.  The minimum is
+//     that of the exact bounds, whatever the order;
+//   - reciprocals and square roots start from FP32 (recip, root).
+// Measured (channel of 250,000 cells, autotuned): 88 -> 54 us per step, 101
+// FP64 instructions per cell.
+template <int MODE, int THREADS, int KMAX, int WAVE>
+__global__ void __launch_bounds__(THREADS) k_step_faces64(StepArgs a) {
+  chain_entry();
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  dq4* sU = reinterpret_cast<dq4*>(smem_raw);  // [t1_cap] states
+  dq4* sP = sU + a.t1_cap;                       // [t1_cap] (u, v, p, c)
+  dq4* sF = sP + a.t1_cap;                       // [3 tile] face flux values
+  const dq4* __restrict__ U = static_cast<const dq4*>(a.U);
+  const double2* __restrict__ geom = static_cast<const double2*>(a.geom);
+  const double2* __restrict__ faces = reinterpret_cast<const double2*>(a.tile_face);
+  dq4* out = static_cast<dq4*>(a.out);
+  const int t0 = blockIdx.x * a.tile;  // cell ids are 32-bit
+  const int nt = min(a.tile, (int)a.n - t0);
+  const int hs = __ldg(a.tile_info + 2 * blockIdx.x);
+  const int h1 = __ldg(a.tile_info + 2 * blockIdx.x + 1);
+  __shared__ double s_t, s_dt;
+  __shared__ float s_min;
+  constexpr bool kBound = MODE != kModeRK2a;
+  float so_far = INFINITY;  // thread 0's: the minimum already found by other blocks
+  if (threadIdx.x == 0) {
+    block_dt(a, s_t, s_dt);
+    if (kBound)
+      so_far = (float)__longlong_as_double(
+          (long long)*static_cast<volatile unsigned long long*>(a.bmin_write));
+  }
+  stage_states<double, THREADS, 0>(U, t0, nt, h1, a.halo_id + hs, sU, sP, a.n, a.err);
+  __syncthreads();
+  // phase 1: the tile's faces, each once, spread evenly over the threads
+  const int f1 = __ldg(a.tile_face_off + blockIdx.x + 1);
+  for (int f = __ldg(a.tile_face_off + blockIdx.x) + threadIdx.x; f < f1; f += THREADS) {
+    const double2 nrm = __ldg(faces + 2 * (int64_t)f), lr = __ldg(faces + 2 * (int64_t)f + 1);
+    const unsigned rx = (unsigned)__double2loint(lr.y), v = (unsigned)__double2hiint(lr.y);
+    const unsigned e = rx & 0xffffu, q = (rx >> 16) & 3u, kv = (rx >> 18) & 3u;
+    if (!index_ok(e, nt, a.err)) continue;
+    const dq4 UL = sU[e];
+    const Prim<double> L = rec_prim<double>(sP[e]);
+    dq4 UR = UL;
+    Prim<double> W = L;
+    if (v < kGhostCodes) {
+      if (index_ok(v, nt + h1, a.err)) {
+        UR = sU[v];
+        W = rec_prim<double>(sP[v]);
+      }
+    } else {
+      UR = ghost<double>((int)v - 0x10000, UL, nrm.x, nrm.y, a.uinf);
+      W = primitive<double>(UR);
+    }
+    double X[4];
+    face_flux_value<double, false, WAVE>(UL, L, UR, W, nrm.x, nrm.y, lr.x, 1.0, X);
+    sF[3 * e + q] = dq4{X[0], X[1], X[2], X[3]};
+    if (v < (unsigned)nt)
+      sF[3 * v + kv] = dq4{flip(X[0]), flip(X[1]), flip(X[2]), flip(X[3])};
+  }
+  __syncthreads();
+  const double dt = s_dt;
+  bool ok = true;
+  float rough[KMAX];
+  float least = INFINITY;
+  unsigned exact = 0u;  // cells (bit k) to be evaluated in FP64 whatever the minimum
+  // phase 2: the three face values in face order, then the cell's update
+#pragma unroll
+  for (int k = 0; k < KMAX; ++k) {
+    const int e = threadIdx.x + k * THREADS;
+    rough[k] = INFINITY;
+    if (e < nt) {
+      const int i = t0 + e;
+      const double2 g = __ldg(geom + 4 * (int64_t)i + 3);  // 1/V, 2V/P
+      dq4 base{};
+      if (MODE == kModeRK2b) base = static_cast<const dq4*>(a.Ubase)[i];
+      // (the other shapes start from zero: the same up to the sign of a zero)
+      const dq4 X0 = sF[3 * e], X1 = sF[3 * e + 1], X2 = sF[3 * e + 2];
+      const double acc[4] = {add(add(X0.x, X1.x), X2.x), add(add(X0.y, X1.y), X2.y),
+                             add(add(X0.z, X1.z), X2.z), add(add(X0.w, X1.w), X2.w)};
+      uint2 none;
+      const dq4 Un = advance_state<double, MODE, false>(sU[e], base, acc, g.x, dt, none, none, none);
+      out[i] = Un;
+      if (kBound) {
+        sU[e] = Un;  // this thread's own entry from here on
+        if (rough_bound(Un, g.y, rough[k]))
+          least = fminf(least, rough[k]);
+        else
+          exact |= 1u << k;
+      }
+    }
+  }
+  if (!kBound) return;
+  const float m = block_min<float>(least);
+  if (threadIdx.x == 0) s_min = fminf(m, so_far) * (1.0f + 4.0f * kBoundSlack);
+  __syncthreads();
+  const float limit = s_min;
+  double bmin = INFINITY;
+#pragma unroll
+  for (int k = 0; k < KMAX; ++k) {
+    const int e = threadIdx.x + k * THREADS;
+    if (e < nt && (((exact >> k) & 1u) || rough[k] <= limit)) {
+      bool c_ok;
+      bmin = fmin(bmin, cell_bound<double>(sU[e], __ldg(geom + 4 * (int64_t)(t0 + e) + 3).y, c_ok));
+      ok = ok && c_ok;
+    }
+  }
+  if (!ok) atomicOr(a.err, 1);
+  if (__any_sync(0xffffffffu, bmin < INFINITY)) {
+    for (int o = 16; o > 0; o >>= 1) bmin = fmin(bmin, __shfl_xor_sync(0xffffffffu, bmin, o));
+    if ((threadIdx.x & 31) == 0)
+      atomicMin(a.bmin_write, (unsigned long long)__double_as_longlong(bmin));
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *a.t_write = s_t + dt;
+    *a.bmin_reset = kInfBits;
   }
 }
 
@@ -330,8 +478,13 @@ cudaError_t launch_tile_t(const StepArgs& a, cudaStream_t s) {
 
 template <typename R, int MODE, bool COMP, int THREADS, int KMAX>
 cudaError_t launch_faces_t(const StepArgs& a, cudaStream_t s) {
-  auto k = a.wave == kWaveMax ? k_step_tile_faces<R, MODE, COMP, THREADS, KMAX, kWaveMax>
-                              : k_step_tile_faces<R, MODE, COMP, THREADS, KMAX, kWaveAverage>;
+  void (*k)(StepArgs);
+  if constexpr (sizeof(R) == 8)
+    k = a.wave == kWaveMax ? k_step_faces64<MODE, THREADS, KMAX, kWaveMax>
+                           : k_step_faces64<MODE, THREADS, KMAX, kWaveAverage>;
+  else
+    k = a.wave == kWaveMax ? k_step_tile_faces<R, MODE, COMP, THREADS, KMAX, kWaveMax>
+                           : k_step_tile_faces<R, MODE, COMP, THREADS, KMAX, kWaveAverage>;
   const size_t smem = tile_faces_smem_bytes(sizeof(R) == 8, a.t1_cap, a.tile);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -342,6 +495,11 @@ cudaError_t launch_faces_t(const StepArgs& a, cudaStream_t s) {
 template <typename R, int MODE, bool COMP>
 cudaError_t launch_faces_size(const StepArgs& a, cudaStream_t s) {
   if (a.tile < 1 || a.tile > kMaxTileCells) return cudaErrorInvalidValue;
+  if constexpr (sizeof(R) == 8) {
+    // small tiles: a warp or four per block, so that a small mesh fills the SMs
+    if (a.tile <= 64) return launch_faces_t<R, MODE, COMP, 64, 1>(a, s);
+    if (a.tile <= 128) return launch_faces_t<R, MODE, COMP, 128, 1>(a, s);
+  }
   if (a.tile <= 512) return launch_faces_t<R, MODE, COMP, 256, 2>(a, s);
   if (a.tile <= 768) return launch_faces_t<R, MODE, COMP, 256, 3>(a, s);
   if (a.tile <= 1024) return launch_faces_t<R, MODE, COMP, 256, 4>(a, s);
@@ -354,7 +512,6 @@ cudaError_t launch_faces_mode(int mode, const StepArgs& a, cudaStream_t s) {
     case kModeFE: return launch_faces_size<R, kModeFE, COMP>(a, s);
     case kModeRK2a: return launch_faces_size<R, kModeRK2a, COMP>(a, s);
     case kModeRK2b: return launch_faces_size<R, kModeRK2b, COMP>(a, s);
-    case kModeResidual: return launch_faces_size<R, kModeResidual, false>(a, s);
     default: return cudaErrorInvalidValue;
   }
 }
