@@ -146,6 +146,7 @@ struct fv_mesh {
   int* d_face_off = nullptr;   // shape 7: the faces each tile evaluates once
   uint2* d_face_rec = nullptr;
   int p_e_cap = 0, p_t1_cap = 0;
+  bool tiles_quick = false;  // FP32: the one-step tiles are all resident at a time
   // normals from vertex coordinates (fv_mesh_set_geometry): tile nodes
   int geometry = FV_GEOM_STORED;
   bool tiles_vertex = false;  // the tile arrays above carry the vertex layout
@@ -350,6 +351,7 @@ void ensure_tiles(fv_mesh* m, cudaStream_t s) {
   FV_CUDA(cudaStreamSynchronize(s));  // L is a local staging buffer
   m->p_e_cap = L.e_cap;
   m->p_t1_cap = L.t1_cap;
+  m->tiles_quick = !m->f64() && fv::tile_quick_fits(m->h.n, m->pair_tile, L.t1_cap);
   m->p_v_cap = V.v_cap;
   m->tiles_vertex = m->vertex_tiles();
   m->tiles_built = m->pair_tile;
@@ -566,6 +568,7 @@ fv::StepArgs base_args(const fv_mesh* m) {
     a.halo_id = m->d_halo_id;
     a.tile = m->tiles_built;
     a.t1_cap = m->p_t1_cap;
+    a.quick = m->tiles_quick;
     a.tile_face_off = m->d_face_off;
     a.tile_face = m->d_face_rec;
     if (m->tiles_vertex) {

@@ -390,10 +390,11 @@ struct CellIn {
   uint2 lo, lo_stage;
 };
 
-template <typename R, int MODE, bool COMP>
-__device__ __forceinline__ void load_cell(const StepArgs& a, const rec_t<R>* __restrict__ U,
-                                          const rec_t<R>* __restrict__ geom, int64_t i,
-                                          CellIn<R>& c) {
+// load_tables: what no step writes (geometry and neighbour ids; may be read
+// before the previous step's kernel has ended); load_values: the rest.
+template <typename R>
+__device__ __forceinline__ void load_tables(const StepArgs& a, const rec_t<R>* __restrict__ geom,
+                                            int64_t i, CellIn<R>& c) {
   c.g0 = Rec<R>::ld(geom + 2 * i);
   c.g1 = Rec<R>::ld(geom + 2 * i + 1);
   if constexpr (sizeof(R) == 8) {
@@ -403,12 +404,25 @@ __device__ __forceinline__ void load_cell(const StepArgs& a, const rec_t<R>* __r
     const int2 nb = __ldg(static_cast<const int2*>(a.nbr) + i);
     c.n0 = __float_as_int(c.g1.w), c.n1 = nb.x, c.n2 = nb.y;
   }
+}
+
+template <typename R, int MODE, bool COMP>
+__device__ __forceinline__ void load_values(const StepArgs& a, const rec_t<R>* __restrict__ U,
+                                            int64_t i, CellIn<R>& c) {
   c.U = Rec<R>::ld(U + i);
   // plain loads: Ubase and the remainders are rewritten in this kernel (each
   // only by the thread of its own cell)
   if (MODE == kModeRK2b) c.base = static_cast<const rec_t<R>*>(a.Ubase)[i];
   if (COMP && MODE != kModeResidual) c.lo = a.lo[i];
   if (COMP && MODE == kModeRK2b) c.lo_stage = a.lo_stage[i];
+}
+
+template <typename R, int MODE, bool COMP>
+__device__ __forceinline__ void load_cell(const StepArgs& a, const rec_t<R>* __restrict__ U,
+                                          const rec_t<R>* __restrict__ geom, int64_t i,
+                                          CellIn<R>& c) {
+  load_tables<R>(a, geom, i, c);
+  load_values<R, MODE, COMP>(a, U, i, c);
 }
 
 // 2V/P of a cell: stored for FP64, from the face lengths for FP32

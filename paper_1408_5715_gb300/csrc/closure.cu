@@ -307,7 +307,6 @@ __device__ __forceinline__ void load_face(const StepArgs& a, const FaceRec* face
 __global__ void __launch_bounds__(kClThreads) k_face_scales(StepArgs a, const FaceRec* faces,
                                                             int64_t nf, ClosureParams cp,
                                                             float* s_cf) {
-  chain_entry();
   __shared__ ClShared sh;
   load_small_params(cp, sh);
   ClFrag fr;
@@ -316,6 +315,7 @@ __global__ void __launch_bounds__(kClThreads) k_face_scales(StepArgs a, const Fa
   ClWarpSmem& w = sh.warp[warp];
   const int64_t wstride = (int64_t)gridDim.x * kClWarps * 32;
   int64_t row = ((int64_t)blockIdx.x * kClWarps + warp) * 32 + lane;
+  chain_entry();
   // this round's face and, issued before this round computes, the next's
   FaceIn cur, nxt;
   for (int64_t base = row - lane; base < nf; base += wstride, row += wstride) {
@@ -613,12 +613,10 @@ __global__ void __launch_bounds__(kTcRows) k_face_scales_tc(StepArgs a, const Fa
 
 template <int MODE, bool COMP>
 __global__ void __launch_bounds__(kBlock) k_step_scaled(StepArgs a, const float* s_cf) {
-  chain_entry();
   const float4* __restrict__ U = static_cast<const float4*>(a.U);
   const float4* __restrict__ geom = static_cast<const float4*>(a.geom);
   float4* out = static_cast<float4*>(a.out);
-  double t = 0.0, dt = 0.0;
-  if (MODE != kModeResidual) dt = step_dt(a, t);
+  __shared__ double s_t, s_dt;
   float bmin = INFINITY;
   bool ok = true;
   const int n = (int)a.n;
@@ -626,11 +624,17 @@ __global__ void __launch_bounds__(kBlock) k_step_scaled(StepArgs a, const float*
   CellIn<float> cur, nxt;
   float sc[3], sn[3];  // the scales of the cell, and of the next (loaded with its records)
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  // as k_step: the first cell's tables before the wait, dt once per block
+  if (i < n) load_tables<float>(a, geom, i, cur);
+  chain_entry();
   if (i < n) {
-    load_cell<float, MODE, COMP>(a, U, geom, i, cur);
+    load_values<float, MODE, COMP>(a, U, i, cur);
 #pragma unroll
     for (int k = 0; k < 3; ++k) sc[k] = __ldg(s_cf + 3 * i + k);
   }
+  if (MODE != kModeResidual && threadIdx.x == 0) block_dt(a, s_t, s_dt);
+  if (MODE != kModeResidual) __syncthreads();
+  const double t = MODE != kModeResidual ? s_t : 0.0, dt = MODE != kModeResidual ? s_dt : 0.0;
   for (; i < n; i += stride) {
     const int j = i + stride;
     if (j < n) {
@@ -683,7 +687,6 @@ __global__ void __launch_bounds__(kBlock) k_step_scaled(StepArgs a, const float*
 // ---------------------------------------------------------------------------
 template <int MODE, bool COMP, int THREADS, int KMAX>
 __global__ void __launch_bounds__(THREADS) k_step_closure_tile(StepArgs a, ClosureParams cp) {
-  chain_entry();
   constexpr int kWarps = THREADS / 32;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float4* sU = reinterpret_cast<float4*>(smem_raw);  // [t1_cap] states
@@ -701,6 +704,7 @@ __global__ void __launch_bounds__(THREADS) k_step_closure_tile(StepArgs a, Closu
   const int nt = min(a.tile, (int)a.n - t0);
   const int hs = __ldg(a.tile_info + 2 * blockIdx.x);
   const int h1 = __ldg(a.tile_info + 2 * blockIdx.x + 1);
+  chain_entry();
   __shared__ double s_t, s_dt;
   if (threadIdx.x == 0 && MODE != kModeResidual) block_dt(a, s_t, s_dt);
   stage_states<float, THREADS, kStageBatch<float, KMAX>>(U, t0, nt, h1, a.halo_id + hs, sU, sP,

@@ -98,6 +98,8 @@ struct StepArgs {
   float vscale;
   // launch as part of a programmatic chain (launch_util.cuh)
   bool chained;
+  // shape 6: all tiles are resident at a time (tile_quick_fits)
+  bool quick;
   // kWaveAverage or kWaveMax (shapes 0, 1 and 6; the others run shape 1)
   int wave;
 };
@@ -197,6 +199,8 @@ cudaError_t launch_restrict_mean(bool fine_f64, bool coarse_f64, const void* Uf,
                                  const int* fine_of, int64_t n_coarse, int kids, void* Uc,
                                  cudaStream_t s);
 cudaError_t launch_step_tile(bool f64, int mode, const StepArgs& a, cudaStream_t s);
+constexpr int kQuickTile = 256;  // largest tile of its one-cell-per-thread form
+bool tile_quick_fits(int64_t n, int tile, int t1_cap);
 // shape 7: the tile shape with each face evaluated once (its states and
 // primitives as shape 6, plus three face-flux records per tile cell)
 inline size_t tile_faces_smem_bytes(bool f64, int t1_cap, int tile) {

@@ -177,7 +177,6 @@ __device__ __forceinline__ void pair_finish(const PairArgs& a, float bmin, bool 
 
 template <int THREADS, int KMAX, bool COMP>
 __global__ void __launch_bounds__(THREADS) k_step_pair(PairArgs a) {
-  chain_entry();
   extern __shared__ float4 smem[];
   float4* sU0 = smem;              // [e_cap]  U^n of tile + both halos
   float4* sU1 = smem + a.e_cap;    // [t1_cap] U^{n+1} of tile + first halo
@@ -186,6 +185,7 @@ __global__ void __launch_bounds__(THREADS) k_step_pair(PairArgs a) {
   const int hs = __ldg(a.tile_info + 2 * blockIdx.x);
   const int h1 = __ldg(a.tile_info + 2 * blockIdx.x + 1);
   const int h12 = __ldg(a.tile_info + 2 * blockIdx.x + 2) - hs;  // both halos
+  chain_entry();
   __shared__ PairDt sdt;
   if (threadIdx.x == 0) pair_dt(a, sdt);
 

@@ -31,7 +31,6 @@ namespace {
 template <typename R, int MODE, bool COMP, int THREADS, int KMAX, int WAVE, bool VTX>
 __global__ void __launch_bounds__(THREADS, sizeof(R) == 4 ? 1280 / THREADS : 1)
     k_step_tile(StepArgs a) {
-  chain_entry();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   rec_t<R>* sU = reinterpret_cast<rec_t<R>*>(smem_raw);  // [t1_cap] states
   rec_t<R>* sP = sU + a.t1_cap;                            // [t1_cap] (u, v, p, c)
@@ -43,6 +42,7 @@ __global__ void __launch_bounds__(THREADS, sizeof(R) == 4 ? 1280 / THREADS : 1)
   const int nt = min(a.tile, (int)a.n - t0);
   const int hs = __ldg(a.tile_info + 2 * blockIdx.x);
   const int h1 = __ldg(a.tile_info + 2 * blockIdx.x + 1);
+  chain_entry();
   // dt formed once per block (FP64 scalar work), read after the barrier
   __shared__ double s_t, s_dt;
   if (threadIdx.x == 0 && MODE != kModeResidual) block_dt(a, s_t, s_dt);
@@ -114,6 +114,104 @@ __global__ void __launch_bounds__(THREADS, sizeof(R) == 4 ? 1280 / THREADS : 1)
   }
 }
 
+// The tile shape for tiles that are all resident at a time, one cell per
+// thread (FP32, up to kQuickTile cells).  A step of such a mesh (some 12,000 to
+// 150,000 cells) is a chain of latencies, so what does not depend on the
+// previous step is done while that still runs: the kernel lets its successor
+// start at once (griddepcontrol.launch_dependents; the successor's blocks fit
+// beside it), which loads the tile's tables and its threads' geometry and then
+// waits for this grid's end.  One warp forms dt (FP64, some 400 clocks) while
+// the others load states, form primitives and sum fluxes.
+// Measured (us per step, compensated, tiles of 128; k_step_tile -> this):
+// 16,384 cells 2.67 -> 2.08, 41,410 2.98 -> 2.30, 65,536 3.23 -> 2.47.
+__device__ __forceinline__ void compute_sync(int threads) {
+  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+
+template <int MODE, bool COMP, int WAVE>
+__global__ void __launch_bounds__(kQuickTile + 32, 4) k_step_tile_quick(StepArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  float4* sU = reinterpret_cast<float4*>(smem_raw);  // [t1_cap] states
+  float4* sP = sU + a.t1_cap;                          // [t1_cap] (u, v, p, c)
+  __shared__ float s_dt, s_min[kQuickTile / 32];
+  const int threads = blockDim.x - 32, tid = threadIdx.x, lane = tid & 31;
+  constexpr bool kBound = MODE != kModeRK2a;
+  if (tid >= threads) {  // the warp of dt
+    chain_entry();
+    chain_next();
+    double t, dt;
+    block_dt(a, t, dt);
+    if (lane == 0) s_dt = (float)dt;
+    __syncthreads();
+    if (!kBound) return;
+    if (blockIdx.x == 0 && lane == 0) {
+      *a.t_write = t + dt;
+      *a.bmin_reset = kInfBits;
+    }
+    __syncthreads();  // the warps' minima are there
+    float m = lane < threads / 32 ? s_min[lane] : INFINITY;
+    m = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(m)));  // positive or inf
+    if (lane == 0) atomicMin(a.bmin_write, (unsigned long long)__double_as_longlong((double)m));
+    return;
+  }
+  const float4* __restrict__ geom = static_cast<const float4*>(a.geom);
+  const float4* U = static_cast<const float4*>(a.U);  // written by the previous grid
+  float4* out = static_cast<float4*>(a.out);
+  const int t0 = blockIdx.x * a.tile;
+  const int nt = min(a.tile, (int)a.n - t0);
+  const int hs = __ldg(a.tile_info + 2 * blockIdx.x);
+  const int h1 = __ldg(a.tile_info + 2 * blockIdx.x + 1);
+  const int i = t0 + tid;
+  const bool has = tid < nt;
+  CellIn<float> c{};
+  uint2 ln = make_uint2(0u, 0u);
+  if (has) {
+    c.g0 = __ldg(geom + 2 * i);
+    c.g1 = __ldg(geom + 2 * i + 1);
+    ln = __ldg(a.cell_ln + i);
+  }
+  int g = tid < h1 ? __ldg(a.halo_id + hs + tid) : 0;
+  if (!index_ok(g, a.n, a.err)) g = t0;
+  chain_entry();
+  chain_next();
+  if (has) {
+    c.U = U[i];
+    if (MODE == kModeRK2b) c.base = static_cast<const float4*>(a.Ubase)[i];
+    if (COMP) c.lo = a.lo[i];
+    if (COMP && MODE == kModeRK2b) c.lo_stage = a.lo_stage[i];
+  }
+  float4 halo = make_float4(1.f, 0.f, 0.f, 1.f);
+  if (tid < h1) halo = U[g];
+  Prim<float> L{};
+  if (has) {
+    L = primitive<float>(c.U);
+    sU[tid] = c.U;
+    sP[tid] = prim_rec<float>(L);
+  }
+  if (tid < h1) {
+    sU[nt + tid] = halo;
+    sP[nt + tid] = prim_rec<float>(primitive<float>(halo));
+  }
+  for (int e = tid + threads; e < h1; e += threads) {  // a ring larger than the tile
+    const float4 u = U[staged_id<float>(t0, nt, nt + e, a.halo_id + hs, a.n, a.err)];
+    sU[nt + e] = u;
+    sP[nt + e] = prim_rec<float>(primitive<float>(u));
+  }
+  compute_sync(threads);
+  float acc[4] = {0.f, 0.f, 0.f, 0.f}, perim = 0.f;
+  if (has)
+    perim = cell_fluxes<float, WAVE>(c.g0, c.g1, ln, c.U, L, sU, sP, a.uinf_f, acc, nt + h1, a.err);
+  __syncthreads();  // dt is there
+  bool ok = true;
+  float bmin = INFINITY;
+  if (has) finish_cell<float, MODE, COMP>(a, out, i, c, acc, perim, s_dt, bmin, ok);
+  if (!kBound) return;
+  if (!ok) atomicOr(a.err, 1);
+  bmin = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(bmin)));
+  if (lane == 0) s_min[tid >> 5] = bmin;
+  __syncthreads();
+}
+
 // Shape 7: the tile shape with each face evaluated once.  Phase 1: the
 // threads share the tile's face list (tiles.cpp): every face of a tile cell
 // except those whose other side is a tile cell of lower local id (for a cell
@@ -129,7 +227,6 @@ __global__ void __launch_bounds__(THREADS, sizeof(R) == 4 ? 1280 / THREADS : 1)
 template <typename R, int MODE, bool COMP, int THREADS, int KMAX, int WAVE>
 __global__ void __launch_bounds__(THREADS, 1) k_step_tile_faces(StepArgs a) {
   static_assert(sizeof(R) == 4);
-  chain_entry();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   rec_t<R>* sU = reinterpret_cast<rec_t<R>*>(smem_raw);  // [t1_cap] states
   rec_t<R>* sP = sU + a.t1_cap;                            // [t1_cap] (u, v, p, c)
@@ -141,6 +238,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_tile_faces(StepArgs a) {
   const int nt = min(a.tile, (int)a.n - t0);
   const int hs = __ldg(a.tile_info + 2 * blockIdx.x);
   const int h1 = __ldg(a.tile_info + 2 * blockIdx.x + 1);
+  chain_entry();
   __shared__ double s_t, s_dt;
   if (threadIdx.x == 0 && MODE != kModeResidual) block_dt(a, s_t, s_dt);
   stage_states<R, THREADS, kStageBatch<R, KMAX>>(U, t0, nt, h1, a.halo_id + hs, sU, sP, a.n,
@@ -263,7 +361,6 @@ __device__ __forceinline__ bool rough_bound(const dq4& U, double inradius, float
 // FP64 instructions per cell.
 template <int MODE, int THREADS, int KMAX, int WAVE>
 __global__ void __launch_bounds__(THREADS) k_step_faces64(StepArgs a) {
-  chain_entry();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   dq4* sU = reinterpret_cast<dq4*>(smem_raw);  // [t1_cap] states
   dq4* sP = sU + a.t1_cap;                       // [t1_cap] (u, v, p, c)
@@ -276,6 +373,7 @@ __global__ void __launch_bounds__(THREADS) k_step_faces64(StepArgs a) {
   const int nt = min(a.tile, (int)a.n - t0);
   const int hs = __ldg(a.tile_info + 2 * blockIdx.x);
   const int h1 = __ldg(a.tile_info + 2 * blockIdx.x + 1);
+  chain_entry();
   __shared__ double s_t, s_dt;
   __shared__ float s_min;
   constexpr bool kBound = MODE != kModeRK2a;
@@ -378,7 +476,6 @@ __global__ void __launch_bounds__(THREADS) k_step_faces64(StepArgs a) {
 // first tile advances its time and clears its next slot.
 template <typename R, int MODE, bool COMP, int THREADS, int KMAX>
 __global__ void __launch_bounds__(THREADS) k_step_tile_batch(BatchArgs b) {
-  chain_entry();
   const StepArgs& a = b.s;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   rec_t<R>* sU = reinterpret_cast<rec_t<R>*>(smem_raw);  // [t1_cap] states
@@ -392,6 +489,7 @@ __global__ void __launch_bounds__(THREADS) k_step_tile_batch(BatchArgs b) {
   const int nt = __ldg(b.tile_cells + tile);
   const int hs = __ldg(a.tile_info + 2 * tile);
   const int h1 = __ldg(a.tile_info + 2 * tile + 1);
+  chain_entry();
   __shared__ double s_t, s_dt;
   if (threadIdx.x == 0 && MODE != kModeResidual) {
     const double t = b.t[b.t_read * b.n_meshes + m];
@@ -516,11 +614,22 @@ cudaError_t launch_faces_mode(int mode, const StepArgs& a, cudaStream_t s) {
   }
 }
 
+template <int MODE, bool COMP>
+cudaError_t launch_quick(const StepArgs& a, cudaStream_t s) {
+  auto k = a.wave == kWaveMax ? k_step_tile_quick<MODE, COMP, kWaveMax>
+                              : k_step_tile_quick<MODE, COMP, kWaveAverage>;
+  const unsigned tiles = (unsigned)((a.n + a.tile - 1) / a.tile);
+  return launch_chained(k, tiles, (unsigned)((a.tile + 31) / 32 * 32 + 32),
+                        tile_smem_bytes(false, a.t1_cap), s, a.chained, a);
+}
+
 // Any tile size up to 2048 cells: the block shape whose KMAX x THREADS cells
 // cover it (the cells of a tile beyond nt are skipped).
 template <typename R, int MODE, bool COMP, bool VTX>
 cudaError_t launch_tile_size(const StepArgs& a, cudaStream_t s) {
   if (a.tile < 1 || a.tile > kMaxTileCells) return cudaErrorInvalidValue;
+  if constexpr (sizeof(R) == 4 && !VTX && MODE != kModeResidual)
+    if (a.quick) return launch_quick<MODE, COMP>(a, s);
   if (a.tile <= 512) return launch_tile_t<R, MODE, COMP, 256, 2, VTX>(a, s);
   if (a.tile <= 768) return launch_tile_t<R, MODE, COMP, 256, 3, VTX>(a, s);
   if (a.tile <= 1024) return launch_tile_t<R, MODE, COMP, 256, 4, VTX>(a, s);
@@ -539,6 +648,22 @@ cudaError_t launch_tile_mode(int mode, const StepArgs& a, cudaStream_t s) {
 }
 
 }  // namespace
+
+// Whether all tiles are resident at a time in the one-cell-per-thread form
+// (with the most registers its kernels take, and shared memory without opting
+// in to more).
+bool tile_quick_fits(int64_t n, int tile, int t1_cap) {
+  if (tile > kQuickTile) return false;
+  const int threads = (tile + 31) / 32 * 32 + 32;
+  const size_t smem = tile_smem_bytes(false, t1_cap);
+  int dev = 0, sms = 0, per_sm = 0;
+  if (smem > 48 * 1024 - 512 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &per_sm, k_step_tile_quick<kModeRK2b, true, kWaveAverage>, threads, smem) != cudaSuccess)
+    return false;
+  return (n + tile - 1) / tile <= (int64_t)sms * per_sm;
+}
 
 cudaError_t launch_batch_step_tile(bool f64, int mode, const BatchArgs& b, cudaStream_t s) {
   if (b.n_tiles <= 0) return cudaSuccess;
