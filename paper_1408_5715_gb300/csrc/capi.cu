@@ -131,6 +131,14 @@ struct fv_mesh {
   bool compensated = true;      // FP32 meshes only
   void* user_lo = nullptr;      // caller-owned remainder (fv_mesh_set_remainder)
   int variant = 1;              // step-kernel shape (fv_mesh_autotune / fv_mesh_set_variant)
+  // While no shape was chosen (and one step runs per launch) the library takes
+  // one by the mesh's size (choose_shape, when the device arrays are made).
+  bool shape_chosen = false;
+  int auto_variant = 1, auto_tile = 0;
+  int shape() const { return shape_chosen || blocking == 2 ? variant : auto_variant; }
+  int shape_tile() const {
+    return shape_chosen || blocking == 2 || auto_tile == 0 ? pair_tile : auto_tile;
+  }
   // two steps per launch (fv_mesh_set_blocking): tiles and halos on the device
   int blocking = 1;
   int pair_tile = 1024;
@@ -139,13 +147,19 @@ struct fv_mesh {
   int wave = FV_WAVE_AVERAGE;  // wave speed of the dissipation (fv_mesh_set_wave_speed)
   int closure_engine = FV_CLOSURE_MMA_SYNC;  // fv_mesh_set_closure_engine
   int tiles_built = 0;  // tile size of the arrays below (0: none)
+  unsigned char* d_tiles_mem = nullptr;  // holds the tiles' arrays
+  unsigned char* d_faces_mem = nullptr;  // holds the arrays of shape 7's faces
   uint2* d_cell_ln = nullptr;
   int* d_tile_info = nullptr;
   int* d_halo_id = nullptr;
   uint2* d_halo_ln = nullptr;
   int* d_face_off = nullptr;   // shape 7: the faces each tile evaluates once
   uint2* d_face_rec = nullptr;
+  uint2* d_cell_ref = nullptr;  // FP64: where a cell's faces are in its tile's list
+  int p_f_cap = 0;
   int p_e_cap = 0, p_t1_cap = 0;
+  bool tiles_pairs = false;        // the tiles have their second halos
+  int64_t tiles_halo_cells = 0;    // halo entries of all tiles
   bool tiles_quick = false;  // FP32: the one-step tiles are all resident at a time
   // normals from vertex coordinates (fv_mesh_set_geometry): tile nodes
   int geometry = FV_GEOM_STORED;
@@ -211,16 +225,14 @@ struct fv_mesh {
   }
 
   void free_tiles() {
-    dev_free(d_face_off);
-    dev_free(d_face_rec);
-    dev_free(d_cell_ln);
-    dev_free(d_tile_info);
-    dev_free(d_halo_id);
-    dev_free(d_halo_ln);
-    dev_free(d_cell_vl);
-    dev_free(d_tile_voff);
-    dev_free(d_tile_vq);
-    dev_free(d_inv_vol);
+    dev_free(d_faces_mem);
+    dev_free(d_tiles_mem);
+    d_face_off = nullptr;
+    d_face_rec = d_cell_ref = d_cell_ln = d_halo_ln = nullptr;
+    d_tile_info = d_halo_id = d_tile_voff = nullptr;
+    d_cell_vl = nullptr;
+    d_tile_vq = nullptr;
+    d_inv_vol = nullptr;
     tiles_built = 0;
     tiles_vertex = false;
     p_v_cap = 0;
@@ -264,97 +276,115 @@ namespace {
 // Tiles and halos of the two-step update, built on the host for the current
 // numbering and tile size and copied to the device.
 bool tiled_shape(int v) { return v == fv::kTileVariant || v == fv::kFaceTileVariant; }
-bool uses_tiles(const fv_mesh* m) { return m->blocking == 2 || tiled_shape(m->variant); }
+bool uses_tiles(const fv_mesh* m) { return m->blocking == 2 || tiled_shape(m->shape()); }
+
+// Several host arrays for one device allocation and one copy.
+struct Staging {
+  std::vector<unsigned char> host;
+  size_t base;  // bytes of the allocation before the copied part
+  explicit Staging(size_t base_bytes = 0) : base((base_bytes + 255) / 256 * 256) {}
+  // Appends v (16-byte aligned, at least `at_least` bytes); its offset in the allocation.
+  template <typename V>
+  size_t put(const V& v, size_t at_least = 4) {
+    host.resize((host.size() + 15) / 16 * 16);
+    const size_t at = host.size(), bytes = v.size() * sizeof(v[0]);
+    host.resize(at + std::max(bytes, at_least));
+    if (bytes) std::memcpy(host.data() + at, v.data(), bytes);
+    return base + at;
+  }
+  // Allocates and copies (the caller synchronises before this goes).
+  unsigned char* upload(cudaStream_t s) {
+    unsigned char* p = nullptr;
+    FV_CUDA(cudaMalloc((void**)&p, base + host.size()));
+    const cudaError_t e = cudaMemcpyAsync(p + base, host.data(), host.size(),
+                                          cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) cudaFree(p);
+    FV_CUDA(e);
+    return p;
+  }
+};
 
 // The faces each tile evaluates once (shape 7), uploaded when that shape
-// first runs on the current tiles: FP32 two words per face (tiles.cpp), FP64
-// the face's normal, its length (as the kernels form it: correctly rounded)
-// and the two words, 32 bytes.
+// first runs on the current tiles: two words per face (tiles.cpp), which FP64
+// meshes expand on the device to 32-byte records with the face's normal and
+// length.
 void upload_tile_faces(fv_mesh* m, const fv::PairTiles& L, cudaStream_t s) {
   const size_t nf = L.face_rec.size() / 2;
-  std::vector<double> rec;
+  Staging st(m->f64() ? std::max<size_t>(nf, 1) * 32 : 0);
+  const size_t off = st.put(L.face_off), words = st.put(L.face_rec, 8);
+  const size_t ref = m->f64() ? st.put(L.cell_ref) : 0;
+  m->d_faces_mem = st.upload(s);
+  m->d_face_off = reinterpret_cast<int*>(m->d_faces_mem + off);
+  m->d_face_rec = reinterpret_cast<uint2*>(m->d_faces_mem + (m->f64() ? 0 : words));
   if (m->f64()) {
-    rec.resize(4 * nf);
-    for (size_t b = 0; b + 1 < L.face_off.size(); ++b)
-      for (int32_t f = L.face_off[b]; f < L.face_off[b + 1]; ++f) {
-        const uint32_t* w = &L.face_rec[2 * (size_t)f];
-        const double* n = &m->h.nrm[2 * (3 * (b * (size_t)L.tile + (w[0] & 0xFFFFu)) +
-                                         ((w[0] >> 16) & 3u))];
-        double* r = &rec[4 * (size_t)f];
-        r[0] = n[0];
-        r[1] = n[1];
-        r[2] = std::sqrt(std::fma(n[0], n[0], n[1] * n[1]));
-        std::memcpy(r + 3, w, 2 * sizeof(uint32_t));
-      }
+    m->d_cell_ref = reinterpret_cast<uint2*>(m->d_faces_mem + ref);
+    m->p_f_cap = L.f_cap;
+    FV_CUDA(fv::launch_face_records(m->d_geom, m->d_face_off,
+                                    reinterpret_cast<const uint2*>(m->d_faces_mem + words),
+                                    (int)L.n_tiles, L.tile, m->d_face_rec, s));
   }
-  const void* src = m->f64() ? static_cast<const void*>(rec.data()) : L.face_rec.data();
-  const size_t bytes = nf * (m->f64() ? 32 : 8);
-  FV_CUDA(cudaMalloc((void**)&m->d_face_off, L.face_off.size() * sizeof(int32_t)));
-  FV_CUDA(cudaMalloc((void**)&m->d_face_rec, std::max<size_t>(bytes, 8)));
-  FV_CUDA(cudaMemcpyAsync(m->d_face_off, L.face_off.data(), L.face_off.size() * sizeof(int32_t),
-                          cudaMemcpyHostToDevice, s));
-  if (bytes) FV_CUDA(cudaMemcpyAsync(m->d_face_rec, src, bytes, cudaMemcpyHostToDevice, s));
-  FV_CUDA(cudaStreamSynchronize(s));  // L and rec are staging buffers
+  FV_CUDA(cudaStreamSynchronize(s));  // L and st are staging buffers
 }
 
 void ensure_tiles(fv_mesh* m, cudaStream_t s) {
   if (!uses_tiles(m) || m->h.n == 0) return;
-  if (m->tiles_built == m->pair_tile && m->tiles_vertex == m->vertex_tiles()) {
-    if (m->variant == fv::kFaceTileVariant && !m->d_face_rec) {
+  const int tile = m->shape_tile();
+  const bool pairs = m->blocking == 2;
+  const bool faces = m->shape() == fv::kFaceTileVariant && !m->vertex_tiles();
+  if (m->tiles_built == tile && m->tiles_vertex == m->vertex_tiles() &&
+      (m->tiles_pairs || !pairs)) {
+    if (faces && !m->d_face_rec) {
       m->drop_graph();
-      upload_tile_faces(m, fv::build_pair_tiles(m->h, m->pair_tile), s);
+      upload_tile_faces(m, fv::build_step_tiles(m->h, tile, true), s);
     }
     return;
   }
   m->free_tiles();
   m->drop_graph();
-  fv::PairTiles L = fv::build_pair_tiles(m->h, m->pair_tile);
-  if (m->variant == fv::kFaceTileVariant && !m->vertex_tiles()) upload_tile_faces(m, L, s);
+  fv::PairTiles L =
+      pairs ? fv::build_pair_tiles(m->h, tile) : fv::build_step_tiles(m->h, tile, faces);
+  if (faces) upload_tile_faces(m, L, s);
   fv::TileVertices V;
   if (m->vertex_tiles()) {
-    V = fv::build_tile_vertices(m->h, m->pair_tile);
+    V = fv::build_tile_vertices(m->h, tile);
     for (int64_t c = 0; c < m->h.n; ++c)  // node 0 replaces the reverse-face bits
       L.cell_ln[2 * c + 1] = (L.cell_ln[2 * c + 1] & 0xFFFFu) | ((uint32_t)V.v0[c] << 16);
     const size_t ncells = (size_t)m->h.n;
-    FV_CUDA(cudaMalloc((void**)&m->d_cell_vl, ncells * sizeof(unsigned)));
-    FV_CUDA(cudaMalloc((void**)&m->d_inv_vol, ncells * sizeof(float)));
     V.inv_vol.resize(ncells);  // the FP32 1/V of the geometry records
     for (size_t c = 0; c < ncells; ++c) V.inv_vol[c] = (float)(1.0 / m->h.vol[c]);
-    FV_CUDA(cudaMemcpyAsync(m->d_inv_vol, V.inv_vol.data(), ncells * sizeof(float),
-                            cudaMemcpyHostToDevice, s));
-    FV_CUDA(cudaMalloc((void**)&m->d_tile_voff, V.voff.size() * sizeof(int32_t)));
-    FV_CUDA(cudaMalloc((void**)&m->d_tile_vq, std::max<size_t>(V.vq.size(), 2) * sizeof(int32_t)));
-    FV_CUDA(cudaMemcpyAsync(m->d_cell_vl, V.cell_vl.data(), ncells * sizeof(unsigned),
-                            cudaMemcpyHostToDevice, s));
-    FV_CUDA(cudaMemcpyAsync(m->d_tile_voff, V.voff.data(), V.voff.size() * sizeof(int32_t),
-                            cudaMemcpyHostToDevice, s));
-    FV_CUDA(cudaMemcpyAsync(m->d_tile_vq, V.vq.data(), V.vq.size() * sizeof(int32_t),
-                            cudaMemcpyHostToDevice, s));
   }
   // whole 256-cell tiles: the staged kernel copies an even number of records
   const size_t ncells = (size_t)((m->h.n + fv::kPadCells - 1) / fv::kPadCells * fv::kPadCells);
-  FV_CUDA(cudaMalloc((void**)&m->d_cell_ln, ncells * sizeof(uint2)));
-  FV_CUDA(cudaMalloc((void**)&m->d_tile_info, L.tile_info.size() * sizeof(int32_t)));
-  const size_t nh = std::max<size_t>(L.halo_id.size(), 1);
-  FV_CUDA(cudaMalloc((void**)&m->d_halo_id, nh * sizeof(int32_t)));
-  FV_CUDA(cudaMalloc((void**)&m->d_halo_ln, nh * sizeof(uint2)));
-  FV_CUDA(cudaMemcpyAsync(m->d_cell_ln, L.cell_ln.data(), L.cell_ln.size() * sizeof(uint32_t),
-                          cudaMemcpyHostToDevice, s));
-  FV_CUDA(cudaMemcpyAsync(m->d_tile_info, L.tile_info.data(), L.tile_info.size() * sizeof(int32_t),
-                          cudaMemcpyHostToDevice, s));
-  if (!L.halo_id.empty()) {
-    FV_CUDA(cudaMemcpyAsync(m->d_halo_id, L.halo_id.data(), L.halo_id.size() * sizeof(int32_t),
-                            cudaMemcpyHostToDevice, s));
-    FV_CUDA(cudaMemcpyAsync(m->d_halo_ln, L.halo_ln.data(), L.halo_ln.size() * sizeof(uint32_t),
-                            cudaMemcpyHostToDevice, s));
+  Staging st;
+  const size_t ln = st.put(L.cell_ln, ncells * sizeof(uint2)), info = st.put(L.tile_info);
+  const size_t halo = st.put(L.halo_id), halo_ln = pairs ? st.put(L.halo_ln, 8) : 0;
+  size_t vl = 0, voff = 0, vq = 0, inv = 0;
+  if (m->vertex_tiles()) {
+    vl = st.put(V.cell_vl);
+    voff = st.put(V.voff);
+    vq = st.put(V.vq, 8);
+    inv = st.put(V.inv_vol);
   }
-  FV_CUDA(cudaStreamSynchronize(s));  // L is a local staging buffer
+  m->d_tiles_mem = st.upload(s);
+  m->d_cell_ln = reinterpret_cast<uint2*>(m->d_tiles_mem + ln);
+  m->d_tile_info = reinterpret_cast<int*>(m->d_tiles_mem + info);
+  m->d_halo_id = reinterpret_cast<int*>(m->d_tiles_mem + halo);
+  if (pairs) m->d_halo_ln = reinterpret_cast<uint2*>(m->d_tiles_mem + halo_ln);
+  if (m->vertex_tiles()) {
+    m->d_cell_vl = reinterpret_cast<unsigned*>(m->d_tiles_mem + vl);
+    m->d_tile_voff = reinterpret_cast<int*>(m->d_tiles_mem + voff);
+    m->d_tile_vq = reinterpret_cast<int2*>(m->d_tiles_mem + vq);
+    m->d_inv_vol = reinterpret_cast<float*>(m->d_tiles_mem + inv);
+  }
+  FV_CUDA(cudaStreamSynchronize(s));  // st is a local staging buffer
   m->p_e_cap = L.e_cap;
   m->p_t1_cap = L.t1_cap;
-  m->tiles_quick = !m->f64() && fv::tile_quick_fits(m->h.n, m->pair_tile, L.t1_cap);
+  m->tiles_quick = !m->f64() && fv::tile_quick_fits(m->h.n, tile, L.t1_cap);
   m->p_v_cap = V.v_cap;
   m->tiles_vertex = m->vertex_tiles();
-  m->tiles_built = m->pair_tile;
+  m->tiles_pairs = pairs;
+  m->tiles_halo_cells = (int64_t)L.halo_id.size();
+  m->tiles_built = tile;
 }
 
 // Shared memory of the one-step tile kernel of this mesh.
@@ -364,8 +394,8 @@ size_t tile_smem(const fv_mesh* m) {
 
 // ... and of the step kernel of the mesh's tiled shape (6 or 7)
 size_t step_tile_smem(const fv_mesh* m) {
-  return m->variant == fv::kFaceTileVariant
-             ? fv::tile_faces_smem_bytes(m->f64(), m->p_t1_cap, m->tiles_built)
+  return m->shape() == fv::kFaceTileVariant
+             ? fv::tile_faces_smem_bytes(m->f64(), m->p_t1_cap, m->tiles_built, m->p_f_cap)
              : tile_smem(m);
 }
 
@@ -380,24 +410,55 @@ void check_tile_smem(const fv_mesh* m, size_t smem) {
             "(Hilbert) or use smaller tiles");
 }
 
+int sm_count() {
+  int dev = 0, sms = 0;
+  FV_CUDA(cudaGetDevice(&dev));
+  FV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  return sms;
+}
+
+// Tiles of shape 7 in FP64: as few as fit, the same number on every SM and all
+// of one size (an SM with one tile more holds the others up), of up to 1,700
+// cells (some 200 KB of shared memory): large tiles have short rings.  us per
+// step with 1 / 2 / 4 tiles per SM: 12,800 cells 6.6 / 6.9 / 8.3, 102,400
+// 22.6 / 23.1 / 24.7, 250,000 47.4 / 48.6 / 49.7; 640,000 with 3 / 4 / 8: 118 /
+// 124 / 121.
+int64_t fp64_tile(int64_t n) {
+  const int64_t sms = sm_count(), per_sm = (n + sms - 1) / sms;
+  const int64_t tiles = (per_sm + 1699) / 1700;
+  return std::max<int64_t>(32, (n + sms * tiles - 1) / (sms * tiles));
+}
+
+// Tiles of the one-wave form of shape 6 (FP32): four on every SM, 128 cells or
+// more (fewer cells only add blocks).
+int64_t quick_tile(int64_t n) {
+  const int64_t slots = 4 * (int64_t)sm_count();
+  return std::max<int64_t>(128, ((n + slots - 1) / slots + 31) / 32 * 32);
+}
+
 // Tile sizes the autotuner times for the one-step tile shape: the standard
 // ones, and on a mesh of a few waves of resident blocks the sizes that fill
 // whole waves (w waves of b blocks per SM), which avoid a last, partly
 // filled wave.
-std::vector<int> tile_candidates(int64_t n) {
+std::vector<int> tile_candidates(const fv_mesh* m) {
+  const int64_t n = m->h.n;
   // small tiles suit shape 7, whose face records take shared memory
   std::vector<int> t = {256, 384};
   t.insert(t.end(), std::begin(fv::kPairTiles), std::end(fv::kPairTiles));
-  int dev = 0, sms = 0;
-  FV_CUDA(cudaGetDevice(&dev));
-  FV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int sms = sm_count();
+  auto add = [&](int64_t c) {
+    if (c >= 32 && c <= fv::kMaxTileCells && std::find(t.begin(), t.end(), (int)c) == t.end())
+      t.push_back((int)c);
+  };
   for (int b : {5, 4, 3, 2})  // resident blocks per SM of the FP32 / FP64 shapes
     for (int w = 1; w <= 3; ++w) {
       const int64_t slots = (int64_t)w * b * sms;
       const int64_t c = ((n + slots - 1) / slots + 31) / 32 * 32;
-      if (c >= 64 && c <= fv::kMaxTileCells && std::find(t.begin(), t.end(), (int)c) == t.end())
-        t.push_back((int)c);
+      if (c >= 64) add(c);
     }
+  add(m->f64() ? fp64_tile(n) : quick_tile(n));
+  if (m->f64())  // whole waves exactly
+    for (int w = 1; w <= 6; ++w) add((n + (int64_t)w * sms - 1) / ((int64_t)w * sms));
   return t;
 }
 
@@ -425,22 +486,11 @@ void build_loop(fv_mesh* m, cudaStream_t s) {
       return;
     }
   }
-  // one allocation and one copy: the geometry in the loop's order, then the tables
-  const size_t geom_bytes = (size_t)n * 2 * sizeof(float4);
-  std::vector<unsigned char> host;
-  auto put = [&](const auto& v, size_t align, size_t at_least) {
-    host.resize((host.size() + align - 1) / align * align);
-    const size_t at = host.size(), bytes = v.size() * sizeof(v[0]);
-    host.resize(at + std::max(bytes, at_least));
-    if (bytes) std::memcpy(host.data() + at, v.data(), bytes);
-    return geom_bytes + at;
-  };
-  const size_t info = put(L.info, 16, fv::kLoopMaxTiles * sizeof(int4));
-  const size_t ln = put(L.cell_ln, 8, 0), ord = put(L.ord, 4, 0);
-  const size_t ring = put(L.ring_id, 4, 4), push = put(L.push, 4, 4);
-  FV_CUDA(cudaMalloc((void**)&m->d_loop, geom_bytes + host.size()));
-  FV_CUDA(cudaMemcpyAsync(m->d_loop + geom_bytes, host.data(), host.size(), cudaMemcpyHostToDevice,
-                          s));
+  // the geometry in the loop's order, then the tables
+  Staging st((size_t)n * 2 * sizeof(float4));
+  const size_t info = st.put(L.info, fv::kLoopMaxTiles * sizeof(int4)), ln = st.put(L.cell_ln);
+  const size_t ord = st.put(L.ord), ring = st.put(L.ring_id), push = st.put(L.push);
+  m->d_loop = st.upload(s);
   m->loop_geom = reinterpret_cast<float4*>(m->d_loop);
   m->loop_info = reinterpret_cast<int4*>(m->d_loop + info);
   m->loop_ln = reinterpret_cast<uint2*>(m->d_loop + ln);
@@ -449,10 +499,46 @@ void build_loop(fv_mesh* m, cudaStream_t s) {
   m->loop_push = reinterpret_cast<unsigned*>(m->d_loop + push);
   FV_CUDA(fv::launch_loop_geometry(static_cast<const float4*>(m->d_geom), m->loop_ord, (int)n,
                                    m->loop_geom, s));
-  FV_CUDA(cudaStreamSynchronize(s));  // host is a local staging buffer
+  FV_CUDA(cudaStreamSynchronize(s));  // st is a local staging buffer
   m->loop_tile = L.tile;
   m->loop_tiles = L.n_tiles;
   m->loop_cap = L.cap;
+}
+
+// The step-kernel shape of a mesh whose shape was not chosen, by size
+// (measured us per step, forward Euler):
+//   FP64: shape 7 (102,400 cells: 24.5 against 52 for shape 1; 12,800: 9.4
+//   against 19.2), whose tiles must be compact: with rings of more than 2.5
+//   times the tile a face evaluated once no longer pays for staging the ring;
+//   FP32: up to 90,000 cells the one-wave tiles (65,536: 2.4 against 2.6 for
+//   shape 0, 102,400: 3.1 against 2.8) when their rings hold less than 3/4 of
+//   the cells, then shape 0 (160,000: 3.5 against 3.9 for shape 1) up to
+//   230,000 (250,000: 5.3 against 4.8), then shape 1.
+void choose_shape(fv_mesh* m, cudaStream_t s) {
+  m->auto_variant = 1;
+  m->auto_tile = 0;
+  const int64_t n = m->h.n;
+  if (m->shape_chosen || m->blocking == 2 || m->loop_tiles > 0 || n == 0) return;
+  const bool tiled = m->f64() || n <= 90000;
+  if (tiled) {
+    m->auto_variant = m->f64() ? fv::kFaceTileVariant : fv::kTileVariant;
+    m->auto_tile = (int)(m->f64() ? fp64_tile(n) : quick_tile(n));
+    bool good = true;
+    try {
+      ensure_tiles(m, s);
+      check_tile_smem(m, step_tile_smem(m));
+    } catch (const fv::Error& e) {
+      if (e.code != FV_EINVAL) throw;
+      good = false;
+    }
+    good = good && (m->f64() ? 2 * m->tiles_halo_cells <= 5 * n
+                             : m->tiles_quick && 4 * m->tiles_halo_cells <= 3 * n);
+    if (good) return;
+    m->auto_variant = 1;
+    m->auto_tile = 0;
+    m->free_tiles();
+  }
+  if (!m->f64() && n <= 230000) m->auto_variant = 0;
 }
 
 void ensure_device(fv_mesh* m, cudaStream_t s) {
@@ -501,6 +587,7 @@ void ensure_device(fv_mesh* m, cudaStream_t s) {
   FV_CUDA(cudaStreamSynchronize(s));
   m->device = dev;
   m->dirty = false;
+  choose_shape(m, s);
   ensure_tiles(m, s);
 }
 
@@ -511,31 +598,41 @@ void ensure_device(fv_mesh* m, cudaStream_t s) {
 // FP32 geometry record rounds it.  The two sides of a face are matched by
 // neighbour id and exactly opposite normals.
 std::vector<fv::FaceRec> closure_faces(const fv::HostMesh& h) {
-  std::vector<fv::FaceRec> f;
-  f.reserve((size_t)(2 * h.n));
-  auto rec = [&](int64_t c, int k, int b) {
-    return fv::FaceRec{(int)(4 * c + k), b, (float)h.nrm[6 * c + 2 * k],
-                       (float)h.nrm[6 * c + 2 * k + 1]};
-  };
-  for (int64_t c = 0; c < h.n; ++c)
-    for (int k = 0; k < 3; ++k) {
-      const int32_t m = h.nbr[3 * c + k];
-      if (m < 0) {
-        f.push_back(rec(c, k, m));
-        continue;
+  const int workers = fv::host_workers(h.n);
+  std::vector<std::vector<fv::FaceRec>> parts(workers);  // of consecutive cells
+  fv::on_host_threads(workers, [&](int w) {
+    std::vector<fv::FaceRec>& f = parts[w];
+    const int64_t c0 = h.n * w / workers, c1 = h.n * (w + 1) / workers;
+    f.reserve((size_t)(2 * (c1 - c0)));
+    auto rec = [&](int64_t c, int k, int b) {
+      return fv::FaceRec{(int)(4 * c + k), b, (float)h.nrm[6 * c + 2 * k],
+                         (float)h.nrm[6 * c + 2 * k + 1]};
+    };
+    for (int64_t c = c0; c < c1; ++c)
+      for (int k = 0; k < 3; ++k) {
+        const int32_t m = h.nbr[3 * c + k];
+        if (m < 0) {
+          f.push_back(rec(c, k, m));
+          continue;
+        }
+        if (m < c) continue;
+        int km = -1;
+        for (int q = 0; q < 3; ++q)
+          if (h.nbr[3 * (int64_t)m + q] == (int32_t)c && !(m == c && q == k) &&
+              h.nrm[6 * (int64_t)m + 2 * q] == -h.nrm[6 * c + 2 * k] &&
+              h.nrm[6 * (int64_t)m + 2 * q + 1] == -h.nrm[6 * c + 2 * k + 1])
+            km = q;
+        if (km < 0) invalid("closure faces: the two sides of a face do not match");
+        if (m == c && km < k) continue;  // a self-face is listed from its lower index
+        f.push_back(rec(c, k, (int)(4 * (int64_t)m + km)));
       }
-      if (m < c) continue;
-      int km = -1;
-      for (int q = 0; q < 3; ++q)
-        if (h.nbr[3 * (int64_t)m + q] == (int32_t)c && !(m == c && q == k) &&
-            h.nrm[6 * (int64_t)m + 2 * q] == -h.nrm[6 * c + 2 * k] &&
-            h.nrm[6 * (int64_t)m + 2 * q + 1] == -h.nrm[6 * c + 2 * k + 1])
-          km = q;
-      if (km < 0) invalid("closure faces: the two sides of a face do not match");
-      if (m == c && km < k) continue;  // a self-face is listed from its lower index
-      f.push_back(rec(c, k, (int)(4 * (int64_t)m + km)));
-    }
-  return f;
+  });
+  std::vector<fv::FaceRec> all;
+  size_t n = 0;
+  for (const auto& f : parts) n += f.size();
+  all.reserve(n);
+  for (const auto& f : parts) all.insert(all.end(), f.begin(), f.end());
+  return all;
 }
 
 void ensure_faces(fv_mesh* m, cudaStream_t s) {
@@ -571,6 +668,8 @@ fv::StepArgs base_args(const fv_mesh* m) {
     a.quick = m->tiles_quick;
     a.tile_face_off = m->d_face_off;
     a.tile_face = m->d_face_rec;
+    a.cell_ref = m->d_cell_ref;
+    a.f_cap = m->p_f_cap;
     if (m->tiles_vertex) {
       a.cell_vl = m->d_cell_vl;
       a.tile_voff = m->d_tile_voff;
@@ -601,7 +700,7 @@ cudaError_t launch_mode(const fv_mesh* m, int mode, const fv::StepArgs& a, const
     if (e != cudaSuccess) return e;
     return fv::launch_step_scaled(mode, a, m->d_scale, s);
   }
-  return fv::launch_step(m->f64(), mode, m->variant, a, s);
+  return fv::launch_step(m->f64(), mode, m->shape(), a, s);
 }
 
 // Enqueues steps j0 .. j0+count-1 of a loop on stream s.
@@ -609,7 +708,7 @@ void enqueue_steps(fv_mesh* m, void* U, int64_t j0, int64_t count, double cfl, d
                    int32_t scheme, cudaStream_t s, const fv_closure* cl = nullptr,
                    bool lo_alt = false) {
   fv::LoopScalars* sc = m->d_scal;
-  if (!cl && tiled_shape(m->variant) && count > 0) check_tile_smem(m, step_tile_smem(m));
+  if (!cl && tiled_shape(m->shape()) && count > 0) check_tile_smem(m, step_tile_smem(m));
   if (cl && m->variant == fv::kFaceTileVariant && count > 0) {
     if (m->tiles_built > 1024) invalid("the learned closure on tiles takes tiles of up to 1024 cells");
     check_tile_smem(m, fv::closure_tile_smem_bytes(m->p_t1_cap, m->tiles_built,
@@ -770,7 +869,7 @@ void capture_graph(fv_mesh* m, void* U, double cfl, double t_stop, int32_t schem
   m->g_closure = cl;
   m->g_closure_version = cl ? cl->version : 0;
   m->g_comp = m->use_lo();
-  m->g_variant = m->variant;
+  m->g_variant = m->shape();
   m->g_blocking = m->blocking;
   m->g_tile = m->tiles_built;
   m->g_staged = m->pair_staged;
@@ -934,6 +1033,7 @@ int fv_mesh_set_variant(fv_mesh* mesh, int32_t variant) {
     if (variant == fv::kFaceTileVariant && mesh->vertex_tiles())
       invalid("normals from node coordinates run the tile shape 6");
     mesh->variant = variant;
+    mesh->shape_chosen = true;
     mesh->loop_wanted = false;
     mesh->drop_graph();
   });
@@ -1033,6 +1133,7 @@ int fv_mesh_set_geometry(fv_mesh* mesh, int32_t form) {
       }
       mesh->geometry = form;
       mesh->variant = fv::kTileVariant;
+      mesh->shape_chosen = true;
       mesh->loop_wanted = false;
     } else {
       invalid("unknown geometry form");
@@ -1103,7 +1204,7 @@ int fv_mesh_autotune(fv_mesh* mesh, const void* U, int32_t scheme, void* stream,
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     double times[fv::kStepVariants];
     const int keep = mesh->variant, keep_tile = mesh->pair_tile;
-    const bool keep_loop = mesh->loop_wanted;
+    const bool keep_loop = mesh->loop_wanted, keep_chosen = mesh->shape_chosen;
     const int blocking = mesh->blocking;
     double loop_us = INFINITY;
     int best_tile[fv::kStepVariants];
@@ -1127,6 +1228,7 @@ int fv_mesh_autotune(fv_mesh* mesh, const void* U, int32_t scheme, void* stream,
         FV_CUDA(cudaEventElapsedTime(&ms, e0, e1));
         return 1e3 * ms / (double)steps;
       };
+      mesh->shape_chosen = true;
       for (int v = 0; v < fv::kStepVariants; ++v) {
         mesh->variant = v;
         if (!tiled_shape(v)) {
@@ -1138,7 +1240,7 @@ int fv_mesh_autotune(fv_mesh* mesh, const void* U, int32_t scheme, void* stream,
         // long-band order) leave that size out
         times[v] = INFINITY;
         if (v == fv::kFaceTileVariant && mesh->vertex_tiles()) continue;
-        for (int tile : tile_candidates(n)) {
+        for (int tile : tile_candidates(mesh)) {
           mesh->pair_tile = tile;
           try {
             ensure_tiles(mesh, s);
@@ -1172,6 +1274,7 @@ int fv_mesh_autotune(fv_mesh* mesh, const void* U, int32_t scheme, void* stream,
       mesh->variant = keep;
       mesh->pair_tile = keep_tile;
       mesh->loop_wanted = keep_loop;
+      mesh->shape_chosen = keep_chosen;
       mesh->blocking = blocking;
       if (e0) cudaEventDestroy(e0);
       if (e1) cudaEventDestroy(e1);
@@ -1237,7 +1340,8 @@ int fv_mesh_debug_set_index(fv_mesh* mesh, int32_t table, int64_t cell, int32_t 
     if (cell < 0 || cell >= mesh->h.n || slot < 0 || slot > 2) invalid("cell or slot out of range");
     cudaStream_t s = as_stream(stream);
     ensure_device(mesh, s);
-    mesh->loop_wanted = false;  // the loop has tables of its own
+    mesh->shape_chosen = true;  // the tables of that shape are the ones changed
+    mesh->loop_wanted = false;
     if (table == 0) {
       // global neighbour ids: FP32 keeps face 0's in the geometry record
       if (mesh->f64()) {
@@ -1317,7 +1421,7 @@ int fv_step(fv_mesh* mesh, void* U, int64_t nsteps, double cfl, double t_stop, i
         if (!mesh->graph || mesh->g_U != U || mesh->g_scheme != scheme || mesh->g_cfl != cfl ||
             mesh->g_tstop != t_stop || mesh->g_closure != closure ||
             mesh->g_closure_version != (closure ? closure->version : 0) ||
-            mesh->g_comp != mesh->use_lo() || mesh->g_variant != mesh->variant ||
+            mesh->g_comp != mesh->use_lo() || mesh->g_variant != mesh->shape() ||
             mesh->g_blocking != mesh->blocking || mesh->g_tile != mesh->tiles_built ||
             mesh->g_staged != mesh->pair_staged || mesh->g_chained != mesh->chained)
           capture_graph(mesh, U, cfl, t_stop, scheme, closure);
@@ -1634,7 +1738,7 @@ void build_batch_tiles(fv_batch* b, fv_mesh* const* meshes) {
       const int64_t off = b->offsets[k];
       b->mesh_first_tile[k] = (int32_t)b->tile_mesh.size();
       if (m->h.n == 0) continue;
-      const fv::PairTiles L = fv::build_pair_tiles(m->h, kBatchTile);
+      const fv::PairTiles L = fv::build_step_tiles(m->h, kBatchTile, false);
       const int64_t hbase = (int64_t)b->halo_id.size();
       if (hbase + (int64_t)L.halo_id.size() > INT32_MAX) invalid("batch halos too large");
       for (int64_t j = 0; j < L.n_tiles; ++j) {

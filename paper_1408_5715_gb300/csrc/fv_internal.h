@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -81,6 +82,11 @@ struct LocalPart {
 PartRange part_range(int64_t n, int32_t nparts, int32_t part);
 LocalPart build_local_part(const HostMesh& m, int32_t nparts, int32_t part);
 
+// Host threads for work on so many cells (some 3,000 a thread, at most 16),
+// and work(0 .. workers - 1) on them; rethrows the first part's exception.
+int host_workers(int64_t cells);
+void on_host_threads(int workers, const std::function<void(int)>& work);
+
 // Tiles and halos of the two-step update (tiles.cpp).  Per tile b:
 // tile_info[2b] = offset of its halos in halo_id, tile_info[2b+1] = size of
 // the first halo; the second halo runs to tile_info[2b+2].  cell_ln (per cell)
@@ -102,8 +108,18 @@ struct PairTiles {
   // cell of the tile), y = the 16-bit local id across (ring or ghost code)
   std::vector<int32_t> face_off;   // [n_tiles + 1]
   std::vector<uint32_t> face_rec;  // [2 faces]
+  // build_step_tiles with faces: where each face of a cell is in its tile's
+  // list, 16 bits each (f0 | f1 << 16, f2), bit 15 set on the side whose flux
+  // is the negated one; and the most faces of a tile
+  std::vector<uint32_t> cell_ref;  // [2 n]
+  int32_t f_cap = 0;
 };
 PairTiles build_pair_tiles(const HostMesh& m, int32_t tile);
+// The same without second halos (halo_ln empty, e_cap = t1_cap) and, unless
+// `faces`, without face lists and the faces pointing back: what the one-step
+// kernels read, built on several host threads; a tile's boundary faces come
+// last in its list.
+PairTiles build_step_tiles(const HostMesh& m, int32_t tile, bool faces);
 
 // Tiles of the resident loop (loop_step.cu): block b keeps the cells
 // [b*tile, min((b+1)*tile, n)) on chip for a whole time loop.  Inside a tile

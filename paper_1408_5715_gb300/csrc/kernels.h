@@ -84,6 +84,10 @@ struct StepArgs {
   // FP64: 32-byte records nx, ny, length and the face's two words)
   const int* tile_face_off;
   const uint2* tile_face;
+  // ... and in FP64 where a cell's faces are in that list (cell_ref of
+  // tiles.cpp), and the most faces of a tile
+  const uint2* cell_ref;
+  int f_cap;
   // Vertex geometry of the tile variant (FP32; vertex_geom.cpp), or nullptr:
   // normals formed from grid coordinates of the tile's nodes and 1/V read
   // from inv_vol instead of the geom records.  tile_vq[2 tile_voff[b] ..]
@@ -202,10 +206,14 @@ cudaError_t launch_step_tile(bool f64, int mode, const StepArgs& a, cudaStream_t
 constexpr int kQuickTile = 256;  // largest tile of its one-cell-per-thread form
 bool tile_quick_fits(int64_t n, int tile, int t1_cap);
 // shape 7: the tile shape with each face evaluated once (its states and
-// primitives as shape 6, plus three face-flux records per tile cell)
-inline size_t tile_faces_smem_bytes(bool f64, int t1_cap, int tile) {
-  return tile_smem_bytes(f64, t1_cap) + (size_t)3 * tile * (f64 ? 32 : 16);
+// primitives as shape 6, plus the flux records: in FP32 three per tile cell, in
+// FP64 one per face, f_cap of them)
+inline size_t tile_faces_smem_bytes(bool f64, int t1_cap, int tile, int f_cap = 0) {
+  return tile_smem_bytes(f64, t1_cap) + (f64 ? (size_t)f_cap * 32 : (size_t)3 * tile * 16);
 }
+// FP64: expands the tiles' face words to 32-byte records (nx, ny, length, words)
+cudaError_t launch_face_records(const void* geom, const int* face_off, const uint2* words,
+                                int n_tiles, int tile, void* records, cudaStream_t s);
 cudaError_t launch_step_tile_faces(bool f64, int mode, const StepArgs& a, cudaStream_t s);
 cudaError_t launch_batch_step_tile(bool f64, int mode, const BatchArgs& b, cudaStream_t s);
 // Library-owned per-cell arrays are allocated in whole tiles of this many

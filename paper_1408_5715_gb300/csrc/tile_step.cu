@@ -23,6 +23,11 @@ namespace fv {
 
 namespace {
 
+// Barrier of a block's compute threads alone (without the warp of dt).
+__device__ __forceinline__ void compute_sync(int threads) {
+  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+
 // VTX (FP32 only): normals from the grid coordinates of the tile's nodes,
 // staged in shared memory after the states (vertex_geom.cpp), and 1/V from a
 // 4-byte array, instead of each cell's 32-byte geometry record.
@@ -124,10 +129,6 @@ __global__ void __launch_bounds__(THREADS, sizeof(R) == 4 ? 1280 / THREADS : 1)
 // the others load states, form primitives and sum fluxes.
 // Measured (us per step, compensated, tiles of 128; k_step_tile -> this):
 // 16,384 cells 2.67 -> 2.08, 41,410 2.98 -> 2.30, 65,536 3.23 -> 2.47.
-__device__ __forceinline__ void compute_sync(int threads) {
-  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
-}
-
 template <int MODE, bool COMP, int WAVE>
 __global__ void __launch_bounds__(kQuickTile + 32, 4) k_step_tile_quick(StepArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -324,48 +325,105 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_tile_faces(StepArgs a) {
   }
 }
 
-// -x without the FP64 pipe.
-__device__ __forceinline__ double flip(double x) {
-  return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x));
+// x with its sign bit changed by `sign` (0 or 0x80000000), without the FP64 pipe.
+__device__ __forceinline__ double flip(double x, unsigned sign) {
+  return __hiloint2double(__double2hiint(x) ^ (int)sign, __double2loint(x));
 }
 
 // A CFL bound in FP32 that rules most cells out of the FP64 minimum: within
 // kBoundSlack of the exact bound of a cell whose state is plainly good (true),
 // else the cell has to be evaluated exactly.
-constexpr float kBoundSlack = 5e-5f;
+constexpr float kBoundSlack = 1e-4f;
+
+// x to float by integer shifts (a conversion takes the FP64 pipe as long as an
+// addition): rounded toward zero, 0 below 2^-100; big is set from 2^100 on.
+__device__ __forceinline__ float rough_float(double x, bool& big) {
+  const unsigned hi = (unsigned)__double2hiint(x), mag = hi & 0x7fffffffu;
+  const unsigned w = __funnelshift_l((unsigned)__double2loint(x), hi, 3);
+  big = big || mag >= (1123u << 20);
+  const unsigned f = ((w ^ 0x40000000u) & 0x7fffffffu) | (hi & 0x80000000u);
+  return mag < (923u << 20) ? 0.0f : __uint_as_float(f);
+}
 
 __device__ __forceinline__ bool rough_bound(const dq4& U, double inradius, float& b) {
-  const float rho = (float)U.x, mx = (float)U.y, my = (float)U.z, E = (float)U.w,
-              r = (float)inradius;
+  bool big = false;
+  const float rho = rough_float(U.x, big), mx = rough_float(U.y, big), my = rough_float(U.z, big),
+              E = rough_float(U.w, big), r = rough_float(inradius, big);
   const float ir = recip<float>(rho), u = mx * ir, v = my * ir;
   const float pe = E - 0.5f * (mx * u + my * v);  // p / (gamma - 1)
   b = r * recip<float>(root<float>(u * u + v * v) +
                        root<float>((float)(kGamma * kGammaM1) * pe * ir));
-  // rounding moves pe by at most a few 2^-24 E: at pe > E / 100 the sound
-  // speed is good to 2e-5, and the exact pressure is positive too
-  return rho > 1e-20f && rho < 1e20f && E < 1e20f && pe > 0.01f * E && pe > 1e-20f && r > 1e-20f;
+  // rounding moves pe by at most a few 2^-23 E: at pe > E / 100 the sound
+  // speed is good to 4e-5, and the exact pressure is positive too
+  return !big && rho > 1e-20f && rho < 1e20f && E < 1e20f && pe > 0.01f * E && pe > 1e-20f &&
+         r > 1e-20f;
 }
 
 // Shape 7 in FP64, bound by the FP64 pipe (two lanes a clock and SM): 84 % of
 // it busy with 173 FP64 instructions per cell in the form above, of which the
 // fluxes are a third.  What is not the fluxes' is taken out:
 //   - a face's record carries its normal and length (32 bytes, read in order),
-//     so no square root per face;
+//     so no square root per face; boundary faces come last in a tile's list,
+//     so that few warps evaluate ghost states; a face's flux is stored once and
+//     the cells find theirs by reference (51 bytes of shared memory a cell
+//     instead of 96 for a slot per side: one more block per SM);
 //   - the CFL bound (two square roots, two divisions) is evaluated only for
 //     cells that may be the minimum: an FP32 bound of every cell, the block's
 //     minimum of those, and FP64 for the cells within the FP32 error of it --
 //     unless the minimum so far already rules the block out.  The minimum is
 //     that of the exact bounds, whatever the order;
 //   - reciprocals and square roots start from FP32 (recip, root).
-// Measured (channel of 250,000 cells, autotuned): 88 -> 54 us per step, 101
-// FP64 instructions per cell.
+// A small mesh is bound by latency instead (a dependent FP64 operation takes
+// 64 clocks): the tile's tables and each thread's first face are read before
+// the previous step ends, the blocks have about a thread per face, and one more
+// warp forms dt.
+// Measured (us per step): channel of 250,000 cells, autotuned, 88 -> 45;
+// square of 12,800 cells 19.2 (shape 1) -> 6.5.
 template <int MODE, int THREADS, int KMAX, int WAVE>
-__global__ void __launch_bounds__(THREADS) k_step_faces64(StepArgs a) {
+__global__ void __launch_bounds__(THREADS + 32) k_step_faces64(StepArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  dq4* sU = reinterpret_cast<dq4*>(smem_raw);  // [t1_cap] states
-  dq4* sP = sU + a.t1_cap;                       // [t1_cap] (u, v, p, c)
-  dq4* sF = sP + a.t1_cap;                       // [3 tile] face flux values
-  const dq4* __restrict__ U = static_cast<const dq4*>(a.U);
+  // 16-byte halves of the records in arrays of their own (no bank conflicts):
+  // states and (u, v, p, c) of tile and ring, flux values of the tile's faces
+  double2* sU[2];
+  double2* sP[2];
+  double2* sF[2];
+  sU[0] = reinterpret_cast<double2*>(smem_raw);
+  sU[1] = sU[0] + a.t1_cap;
+  sP[0] = sU[1] + a.t1_cap;
+  sP[1] = sP[0] + a.t1_cap;
+  sF[0] = sP[1] + a.t1_cap;
+  sF[1] = sF[0] + a.f_cap;
+  auto get = [](double2* const h[2], unsigned e) {
+    const double2 x = h[0][e], y = h[1][e];
+    return dq4{x.x, x.y, y.x, y.y};
+  };
+  auto put = [](double2* const h[2], unsigned e, const dq4& r) {
+    h[0][e] = make_double2(r.x, r.y);
+    h[1][e] = make_double2(r.z, r.w);
+  };
+  __shared__ double s_dt;
+  __shared__ float s_so_far, s_min[THREADS / 32];
+  constexpr bool kBound = MODE != kModeRK2a;
+  const int tid = threadIdx.x;
+  if (tid >= THREADS) {  // the warp of dt
+    chain_entry();
+    double t, dt;
+    block_dt(a, t, dt);
+    if (tid == THREADS) {
+      s_dt = dt;
+      if (kBound)  // the minimum already found by other blocks
+        s_so_far = (float)__longlong_as_double(
+            (long long)*static_cast<volatile unsigned long long*>(a.bmin_write));
+    }
+    __syncthreads();
+    if (kBound && blockIdx.x == 0 && tid == THREADS) {
+      *a.t_write = t + dt;
+      *a.bmin_reset = kInfBits;
+    }
+    if (kBound) __syncthreads();
+    return;
+  }
+  const dq4* U = static_cast<const dq4*>(a.U);  // written by the previous grid
   const double2* __restrict__ geom = static_cast<const double2*>(a.geom);
   const double2* __restrict__ faces = reinterpret_cast<const double2*>(a.tile_face);
   dq4* out = static_cast<dq4*>(a.out);
@@ -373,71 +431,99 @@ __global__ void __launch_bounds__(THREADS) k_step_faces64(StepArgs a) {
   const int nt = min(a.tile, (int)a.n - t0);
   const int hs = __ldg(a.tile_info + 2 * blockIdx.x);
   const int h1 = __ldg(a.tile_info + 2 * blockIdx.x + 1);
-  chain_entry();
-  __shared__ double s_t, s_dt;
-  __shared__ float s_min;
-  constexpr bool kBound = MODE != kModeRK2a;
-  float so_far = INFINITY;  // thread 0's: the minimum already found by other blocks
-  if (threadIdx.x == 0) {
-    block_dt(a, s_t, s_dt);
-    if (kBound)
-      so_far = (float)__longlong_as_double(
-          (long long)*static_cast<volatile unsigned long long*>(a.bmin_write));
-  }
-  stage_states<double, THREADS, 0>(U, t0, nt, h1, a.halo_id + hs, sU, sP, a.n, a.err);
-  __syncthreads();
-  // phase 1: the tile's faces, each once, spread evenly over the threads
+  const int f0 = __ldg(a.tile_face_off + blockIdx.x);
+  int f = f0 + tid;
   const int f1 = __ldg(a.tile_face_off + blockIdx.x + 1);
-  for (int f = __ldg(a.tile_face_off + blockIdx.x) + threadIdx.x; f < f1; f += THREADS) {
-    const double2 nrm = __ldg(faces + 2 * (int64_t)f), lr = __ldg(faces + 2 * (int64_t)f + 1);
-    const unsigned rx = (unsigned)__double2loint(lr.y), v = (unsigned)__double2hiint(lr.y);
-    const unsigned e = rx & 0xffffu, q = (rx >> 16) & 3u, kv = (rx >> 18) & 3u;
+  const int first = tid < nt + h1 ? (int)staged_id<double>(t0, nt, tid, a.halo_id + hs, a.n, a.err) : 0;
+  double2 nrm{}, lr{}, g_first{};
+  if (f < f1) nrm = __ldg(faces + 2 * (int64_t)f), lr = __ldg(faces + 2 * (int64_t)f + 1);
+  uint2 ref_first = make_uint2(0u, 0u);
+  if (tid < nt) {
+    g_first = __ldg(geom + 4 * (int64_t)(t0 + tid) + 3);  // 1/V, 2V/P
+    ref_first = __ldg(a.cell_ref + t0 + tid);
+  }
+  chain_entry();
+  for (int e = tid; e < nt + h1; e += THREADS) {
+    const int64_t i =
+        e == tid ? first : staged_id<double>(t0, nt, e, a.halo_id + hs, a.n, a.err);
+    const double2 x = reinterpret_cast<const double2*>(U + i)[0],
+                  y = reinterpret_cast<const double2*>(U + i)[1];
+    const dq4 u{x.x, x.y, y.x, y.y};
+    put(sU, e, u);
+    put(sP, e, prim_rec<double>(primitive<double>(u)));
+  }
+  compute_sync(THREADS);
+  // phase 1: the tile's faces, each once, spread evenly over the threads, the
+  // next record read ahead
+  while (f < f1) {
+    const double2 n_cur = nrm, l_cur = lr;
+    const int slot = f - f0;
+    f += THREADS;
+    if (f < f1) nrm = __ldg(faces + 2 * (int64_t)f), lr = __ldg(faces + 2 * (int64_t)f + 1);
+    const unsigned rx = (unsigned)__double2loint(l_cur.y), v = (unsigned)__double2hiint(l_cur.y);
+    const unsigned e = rx & 0xffffu;
     if (!index_ok(e, nt, a.err)) continue;
-    const dq4 UL = sU[e];
-    const Prim<double> L = rec_prim<double>(sP[e]);
+    const dq4 UL = get(sU, e);
+    const Prim<double> L = rec_prim<double>(get(sP, e));
     dq4 UR = UL;
     Prim<double> W = L;
     if (v < kGhostCodes) {
       if (index_ok(v, nt + h1, a.err)) {
-        UR = sU[v];
-        W = rec_prim<double>(sP[v]);
+        UR = get(sU, v);
+        W = rec_prim<double>(get(sP, v));
       }
     } else {
-      UR = ghost<double>((int)v - 0x10000, UL, nrm.x, nrm.y, a.uinf);
+      UR = ghost<double>((int)v - 0x10000, UL, n_cur.x, n_cur.y, a.uinf);
       W = primitive<double>(UR);
     }
     double X[4];
-    face_flux_value<double, false, WAVE>(UL, L, UR, W, nrm.x, nrm.y, lr.x, 1.0, X);
-    sF[3 * e + q] = dq4{X[0], X[1], X[2], X[3]};
-    if (v < (unsigned)nt)
-      sF[3 * v + kv] = dq4{flip(X[0]), flip(X[1]), flip(X[2]), flip(X[3])};
+    face_flux_value<double, false, WAVE>(UL, L, UR, W, n_cur.x, n_cur.y, l_cur.x, 1.0, X);
+    put(sF, slot, dq4{X[0], X[1], X[2], X[3]});
   }
   __syncthreads();
   const double dt = s_dt;
   bool ok = true;
+  double2 g[KMAX];
+  uint2 ref[KMAX];
   float rough[KMAX];
   float least = INFINITY;
   unsigned exact = 0u;  // cells (bit k) to be evaluated in FP64 whatever the minimum
+#pragma unroll
+  for (int k = 0; k < KMAX; ++k) {
+    const int e = tid + k * THREADS;
+    g[k] = g_first;
+    ref[k] = ref_first;
+    if (k > 0 && e < nt) {
+      g[k] = __ldg(geom + 4 * (int64_t)(t0 + e) + 3);
+      ref[k] = __ldg(a.cell_ref + t0 + e);
+    }
+  }
   // phase 2: the three face values in face order, then the cell's update
 #pragma unroll
   for (int k = 0; k < KMAX; ++k) {
-    const int e = threadIdx.x + k * THREADS;
+    const int e = tid + k * THREADS;
     rough[k] = INFINITY;
     if (e < nt) {
       const int i = t0 + e;
-      const double2 g = __ldg(geom + 4 * (int64_t)i + 3);  // 1/V, 2V/P
       dq4 base{};
       if (MODE == kModeRK2b) base = static_cast<const dq4*>(a.Ubase)[i];
       // (the other shapes start from zero: the same up to the sign of a zero)
-      const dq4 X0 = sF[3 * e], X1 = sF[3 * e + 1], X2 = sF[3 * e + 2];
+      auto flux = [&](unsigned r) {  // bit 15: the face was evaluated from the other side
+        const unsigned at = r & 0x7fffu, sign = (r & 0x8000u) << 16;
+        const dq4 x = get(sF, index_ok(at, a.f_cap, a.err) ? at : 0u);
+        return dq4{flip(x.x, sign), flip(x.y, sign), flip(x.z, sign), flip(x.w, sign)};
+      };
+      const dq4 X0 = flux(ref[k].x & 0xffffu), X1 = flux(ref[k].x >> 16),
+                X2 = flux(ref[k].y & 0xffffu);
       const double acc[4] = {add(add(X0.x, X1.x), X2.x), add(add(X0.y, X1.y), X2.y),
                              add(add(X0.z, X1.z), X2.z), add(add(X0.w, X1.w), X2.w)};
       uint2 none;
-      const dq4 Un = advance_state<double, MODE, false>(sU[e], base, acc, g.x, dt, none, none, none);
+      const dq4 Un =
+          advance_state<double, MODE, false>(get(sU, e), base, acc, g[k].x, dt, none, none, none);
       out[i] = Un;
       if (kBound) {
-        sU[e] = Un;  // this thread's own entry from here on
-        if (rough_bound(Un, g.y, rough[k]))
+        put(sU, e, Un);  // this thread's own entry from here on
+        if (rough_bound(Un, g[k].y, rough[k]))
           least = fminf(least, rough[k]);
         else
           exact |= 1u << k;
@@ -445,29 +531,41 @@ __global__ void __launch_bounds__(THREADS) k_step_faces64(StepArgs a) {
     }
   }
   if (!kBound) return;
-  const float m = block_min<float>(least);
-  if (threadIdx.x == 0) s_min = fminf(m, so_far) * (1.0f + 4.0f * kBoundSlack);
+  least = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(least)));  // positive
+  if ((tid & 31) == 0) s_min[tid >> 5] = least;
   __syncthreads();
-  const float limit = s_min;
+  least = s_so_far;
+#pragma unroll
+  for (int w = 0; w < THREADS / 32; ++w) least = fminf(least, s_min[w]);
+  const float limit = least * (1.0f + 4.0f * kBoundSlack);
   double bmin = INFINITY;
 #pragma unroll
   for (int k = 0; k < KMAX; ++k) {
-    const int e = threadIdx.x + k * THREADS;
+    const int e = tid + k * THREADS;
     if (e < nt && (((exact >> k) & 1u) || rough[k] <= limit)) {
       bool c_ok;
-      bmin = fmin(bmin, cell_bound<double>(sU[e], __ldg(geom + 4 * (int64_t)(t0 + e) + 3).y, c_ok));
+      bmin = fmin(bmin, cell_bound<double>(get(sU, e), g[k].y, c_ok));
       ok = ok && c_ok;
     }
   }
   if (!ok) atomicOr(a.err, 1);
   if (__any_sync(0xffffffffu, bmin < INFINITY)) {
     for (int o = 16; o > 0; o >>= 1) bmin = fmin(bmin, __shfl_xor_sync(0xffffffffu, bmin, o));
-    if ((threadIdx.x & 31) == 0)
-      atomicMin(a.bmin_write, (unsigned long long)__double_as_longlong(bmin));
+    if ((tid & 31) == 0) atomicMin(a.bmin_write, (unsigned long long)__double_as_longlong(bmin));
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *a.t_write = s_t + dt;
-    *a.bmin_reset = kInfBits;
+}
+
+// The face records of k_step_faces64, a block per tile (once per mesh and tile
+// size); the length is face_len's, as every other kernel forms it.
+__global__ void k_face_records(const dq4* __restrict__ geom, const int* __restrict__ face_off,
+                               const uint2* __restrict__ words, int tile, dq4* records) {
+  const int f1 = face_off[blockIdx.x + 1];
+  for (int f = face_off[blockIdx.x] + threadIdx.x; f < f1; f += blockDim.x) {
+    const uint2 w = words[f];
+    double nx, ny;
+    face_normal<double>(geom, (int)blockIdx.x * tile + (int)(w.x & 0xffffu), (w.x >> 16) & 3u, nx,
+                        ny);
+    records[f] = dq4{nx, ny, face_len<double>(nx, ny), __hiloint2double((int)w.y, (int)w.x)};
   }
 }
 
@@ -583,20 +681,23 @@ cudaError_t launch_faces_t(const StepArgs& a, cudaStream_t s) {
   else
     k = a.wave == kWaveMax ? k_step_tile_faces<R, MODE, COMP, THREADS, KMAX, kWaveMax>
                            : k_step_tile_faces<R, MODE, COMP, THREADS, KMAX, kWaveAverage>;
-  const size_t smem = tile_faces_smem_bytes(sizeof(R) == 8, a.t1_cap, a.tile);
+  const size_t smem = tile_faces_smem_bytes(sizeof(R) == 8, a.t1_cap, a.tile, a.f_cap);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int64_t tiles = (a.n + a.tile - 1) / a.tile;
-  return launch_chained(k, (unsigned)tiles, THREADS, smem, s, a.chained, a);
+  return launch_chained(k, (unsigned)tiles, sizeof(R) == 8 ? THREADS + 32 : THREADS, smem, s,
+                        a.chained, a);
 }
 
 template <typename R, int MODE, bool COMP>
 cudaError_t launch_faces_size(const StepArgs& a, cudaStream_t s) {
   if (a.tile < 1 || a.tile > kMaxTileCells) return cudaErrorInvalidValue;
   if constexpr (sizeof(R) == 8) {
-    // small tiles: a warp or four per block, so that a small mesh fills the SMs
-    if (a.tile <= 64) return launch_faces_t<R, MODE, COMP, 64, 1>(a, s);
-    if (a.tile <= 128) return launch_faces_t<R, MODE, COMP, 128, 1>(a, s);
+    // small tiles: about a thread per face
+    if (a.tile <= 32) return launch_faces_t<R, MODE, COMP, 64, 1>(a, s);
+    if (a.tile <= 64) return launch_faces_t<R, MODE, COMP, 128, 1>(a, s);
+    if (a.tile <= 112) return launch_faces_t<R, MODE, COMP, 192, 1>(a, s);
+    if (a.tile <= 256) return launch_faces_t<R, MODE, COMP, 256, 1>(a, s);
   }
   if (a.tile <= 512) return launch_faces_t<R, MODE, COMP, 256, 2>(a, s);
   if (a.tile <= 768) return launch_faces_t<R, MODE, COMP, 256, 3>(a, s);
@@ -673,11 +774,22 @@ cudaError_t launch_batch_step_tile(bool f64, int mode, const BatchArgs& b, cudaS
   return launch_tile_batch_mode<float, false>(mode, b, s);
 }
 
+cudaError_t launch_face_records(const void* geom, const int* face_off, const uint2* words,
+                                int n_tiles, int tile, void* records, cudaStream_t s) {
+  if (n_tiles <= 0) return cudaSuccess;
+  k_face_records<<<(unsigned)n_tiles, 128, 0, s>>>(static_cast<const dq4*>(geom), face_off, words,
+                                                   tile, static_cast<dq4*>(records));
+  return cudaGetLastError();
+}
+
 cudaError_t launch_step_tile_faces(bool f64, int mode, const StepArgs& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;
   if (!a.cell_ln || !a.tile_info || !a.halo_id || a.tile_vq || !a.tile_face_off || !a.tile_face)
     return cudaErrorInvalidValue;
-  if (f64) return launch_faces_mode<double, false>(mode, a, s);
+  if (f64) {
+    if (!a.cell_ref) return cudaErrorInvalidValue;
+    return launch_faces_mode<double, false>(mode, a, s);
+  }
   if (a.lo) return launch_faces_mode<float, true>(mode, a, s);
   return launch_faces_mode<float, false>(mode, a, s);
 }

@@ -21,6 +21,9 @@
 // the same tile, the face of that neighbour that points back (the tile
 // kernel that evaluates each face once writes the negated flux there).
 #include <algorithm>
+#include <exception>
+#include <functional>
+#include <thread>
 
 #include "fv_internal.h"
 
@@ -134,6 +137,161 @@ PairTiles build_pair_tiles(const HostMesh& m, int32_t tile) {
   L.tile_info[2 * L.n_tiles] = (int32_t)L.halo_id.size();
   L.face_off.push_back((int32_t)(L.face_rec.size() / 2));
   if (L.face_rec.size() / 2 > (size_t)INT32_MAX) throw Error{FV_EINVAL, "too many tile faces"};
+  return L;
+}
+
+namespace {
+
+// Tiles [b0, b1) of build_step_tiles: their parts of tile_info (sizes only)
+// and cell_ln in L, halo ids and faces in order in `part`.
+struct TilePart {
+  std::vector<int32_t> halo, faces_of;  // faces_of: faces of each tile
+  std::vector<uint32_t> face_rec;
+  int32_t t1_cap = 0, f_cap = 0;
+};
+
+void step_tile_range(const HostMesh& m, int32_t tile, bool faces, int32_t b0, int32_t b1,
+                     PairTiles& L, TilePart& part) {
+  std::vector<int32_t> ring;
+  std::vector<uint32_t> ghosts;
+  for (int32_t b = b0; b < b1; ++b) {
+    const int64_t t0 = (int64_t)b * tile, t1 = std::min<int64_t>(t0 + tile, m.n);
+    const int32_t nt = (int32_t)(t1 - t0);
+    ring.clear();
+    for (int64_t j = 3 * t0; j < 3 * t1; ++j) {
+      const int32_t x = m.nbr[j];
+      if (x >= 0 && (x < t0 || x >= t1)) ring.push_back(x);
+    }
+    std::sort(ring.begin(), ring.end());
+    ring.erase(std::unique(ring.begin(), ring.end()), ring.end());
+    if (nt + (int64_t)ring.size() > kLocalLimit)
+      throw Error{FV_EINVAL, "a tile with its halo exceeds 65533 cells; renumber the cells "
+                             "with a compact order (Hilbert) or use smaller tiles"};
+    L.tile_info[2 * b + 1] = (int32_t)ring.size();
+    part.t1_cap = std::max(part.t1_cap, nt + (int32_t)ring.size());
+    part.halo.insert(part.halo.end(), ring.begin(), ring.end());
+    const size_t first_face = part.face_rec.size();
+    for (int64_t c = t0; c < t1; ++c) {
+      const uint32_t e = (uint32_t)(c - t0);
+      uint32_t v[3], back[3] = {0u, 0u, 0u};
+      for (int k = 0; k < 3; ++k) {
+        const int32_t x = m.nbr[3 * c + k];
+        if (x < 0) {
+          v[k] = (uint32_t)(0x10000 + x);
+        } else if (x < t0 || x >= t1) {
+          v[k] = (uint32_t)(nt + (std::lower_bound(ring.begin(), ring.end(), x) - ring.begin()));
+        } else {
+          v[k] = (uint32_t)(x - t0);
+          if (!faces) continue;
+          int kx = -1;  // the face of x that points back
+          for (int q = 0; q < 3; ++q)
+            if (m.nbr[3 * (int64_t)x + q] == (int32_t)c && !(x == c && q == k) &&
+                m.nrm[6 * (int64_t)x + 2 * q] == -m.nrm[6 * c + 2 * k] &&
+                m.nrm[6 * (int64_t)x + 2 * q + 1] == -m.nrm[6 * c + 2 * k + 1])
+              kx = q;
+          if (kx < 0) throw Error{FV_EINVAL, "tile construction: the two sides of a face differ"};
+          back[k] = (uint32_t)kx;
+        }
+      }
+      L.cell_ln[2 * c] = v[0] | (v[1] << 16);
+      L.cell_ln[2 * c + 1] = v[2] | back[0] << 16 | back[1] << 18 | back[2] << 20;
+      if (!faces) continue;
+      for (uint32_t q = 0; q < 3; ++q) {
+        if (v[q] < (uint32_t)nt && (v[q] < e || (v[q] == e && back[q] < q))) continue;
+        std::vector<uint32_t>& list = v[q] < (uint32_t)kLocalLimit ? part.face_rec : ghosts;
+        list.push_back(e | q << 16 | back[q] << 18);
+        list.push_back(v[q]);
+      }
+    }
+    // boundary faces last, so that they fill warps of their own
+    part.face_rec.insert(part.face_rec.end(), ghosts.begin(), ghosts.end());
+    ghosts.clear();
+    const int32_t nf = (int32_t)((part.face_rec.size() - first_face) / 2);
+    part.faces_of.push_back(nf);
+    part.f_cap = std::max(part.f_cap, nf);
+    for (int32_t i = 0; i < nf; ++i) {
+      const uint32_t w = part.face_rec[first_face + 2 * i], v = part.face_rec[first_face + 2 * i + 1];
+      auto refer = [&](uint32_t cell, uint32_t face, uint32_t ref) {
+        L.cell_ref[2 * (t0 + cell) + (face >> 1)] |= ref << (face == 1 ? 16 : 0);
+      };
+      refer(w & 0xFFFFu, (w >> 16) & 3u, (uint32_t)i);
+      if (v < (uint32_t)nt) refer(v, (w >> 18) & 3u, (uint32_t)i | 0x8000u);
+    }
+  }
+}
+
+}  // namespace
+
+int host_workers(int64_t cells) {
+  return (int)std::max<int64_t>(
+      1, std::min<int64_t>({cells / 3000, 16, (int64_t)std::thread::hardware_concurrency()}));
+}
+
+void on_host_threads(int workers, const std::function<void(int)>& work) {
+  std::vector<std::exception_ptr> errors(workers);
+  auto guarded = [&](int w) {
+    try {
+      work(w);
+    } catch (...) {
+      errors[w] = std::current_exception();
+    }
+  };
+  std::vector<std::thread> threads;
+  int started = 1;  // this thread takes the first part, and those no thread could be had for
+  try {
+    threads.reserve(workers);
+    for (; started < workers; ++started) threads.emplace_back(guarded, started);
+  } catch (const std::exception&) {
+  }
+  guarded(0);
+  for (int w = started; w < workers; ++w) guarded(w);
+  for (std::thread& t : threads) t.join();
+  for (const std::exception_ptr& e : errors)
+    if (e) std::rethrow_exception(e);
+}
+
+PairTiles build_step_tiles(const HostMesh& m, int32_t tile, bool faces) {
+  if (tile < 1) throw Error{FV_EINVAL, "tile size must be positive"};
+  if (faces && tile > 10000) throw Error{FV_EINVAL, "tile too large for 15-bit face references"};
+  if (m.n / tile >= INT32_MAX) throw Error{FV_EINVAL, "too many tiles"};
+  PairTiles L;
+  L.tile = tile;
+  L.n_tiles = (m.n + tile - 1) / tile;
+  L.tile_info.assign(2 * (L.n_tiles + 1), 0);
+  L.cell_ln.resize(2 * (size_t)m.n);
+  if (faces) L.cell_ref.assign(2 * (size_t)m.n, 0u);
+  const int workers = host_workers(m.n);
+  std::vector<TilePart> parts(workers);
+  on_host_threads(workers, [&](int w) {
+    step_tile_range(m, tile, faces, (int32_t)(L.n_tiles * w / workers),
+                    (int32_t)(L.n_tiles * (w + 1) / workers), L, parts[w]);
+  });
+  size_t halos = 0, words = 0;
+  for (const TilePart& p : parts) {
+    halos += p.halo.size();
+    words += p.face_rec.size();
+  }
+  if (halos > (size_t)INT32_MAX || words / 2 > (size_t)INT32_MAX)
+    throw Error{FV_EINVAL, "tile halos too large for 32-bit offsets"};
+  L.halo_id.reserve(halos);
+  L.face_rec.reserve(words);
+  int32_t hs = 0, fs = 0, b = 0;
+  for (const TilePart& p : parts) {
+    L.halo_id.insert(L.halo_id.end(), p.halo.begin(), p.halo.end());
+    L.face_rec.insert(L.face_rec.end(), p.face_rec.begin(), p.face_rec.end());
+    L.t1_cap = std::max(L.t1_cap, p.t1_cap);
+    L.f_cap = std::max(L.f_cap, p.f_cap);
+    for (int32_t f : p.faces_of) {
+      L.tile_info[2 * b] = hs;
+      hs += L.tile_info[2 * b + 1];
+      ++b;
+      if (faces) L.face_off.push_back(fs);
+      fs += f;
+    }
+  }
+  L.tile_info[2 * L.n_tiles] = hs;
+  if (faces) L.face_off.push_back(fs);
+  L.e_cap = L.t1_cap;
   return L;
 }
 
