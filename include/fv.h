@@ -203,7 +203,9 @@ int fv_mesh_set_remainder(fv_mesh* mesh, void* lo);
  * slots -- half the face arithmetic, for three flux records per tile cell of
  * shared memory (forward Euler and RK2; the residual runs as shape 0; not
  * with FV_GEOM_VERTEX).  All give bitwise identical results; only speed
- * differs.  FV_EINVAL outside 0..7. */
+ * differs; until one is set (here, by fv_mesh_autotune or by
+ * fv_mesh_set_geometry) the library takes one by the mesh's precision, size and
+ * order, whatever fv_mesh_get_tiling reports.  FV_EINVAL outside 0..7. */
 int fv_mesh_set_variant(fv_mesh* mesh, int32_t variant);
 
 /* Times every step-kernel shape on this mesh (a few steps each on a device
@@ -540,7 +542,9 @@ int fv_batch_info(const fv_batch* batch, int64_t* n_cells_padded, int64_t* offse
  * cells within each mesh with their neighbour ring and primitives in shared
  * memory (needs compactly numbered meshes: FV_EINVAL if a tile's ring does
  * not fit).  Default: 6 when its tiles fit, else 0 (decided at the first
- * device call).  All give bitwise identical results. */
+ * device call); until a shape is set the steps run whichever of 0 and 6 is
+ * quicker for the batch's precision and size.  All give bitwise identical
+ * results. */
 int fv_batch_set_variant(fv_batch* batch, int32_t variant);
 
 /* The batch's kernel shape in *variant: 0, 5 or 6, or -1 while the default

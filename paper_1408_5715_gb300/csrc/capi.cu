@@ -1557,8 +1557,12 @@ struct fv_batch {
   std::vector<double> uinf;          // 4 per mesh (conserved)
   bool compensated = true;
   // 0: one thread per cell; 5: TMA-staged tiles; 6: tiles; -1: 6 when its
-  // tiles fit in shared memory, else 0 (chosen at the first device call)
+  // tiles fit in shared memory, else 0 (at the first device call).  While none
+  // was chosen the steps run the quicker of 0 and 6 (auto_variant).
   int variant = -1;
+  bool shape_chosen = false;
+  int auto_variant = 0;
+  int shape() const { return shape_chosen ? variant : auto_variant; }
   // shared-memory tiles of 1024 cells within each mesh (shape 6)
   bool tiles_ok = false;
   int32_t t1_cap = 0;
@@ -1724,6 +1728,11 @@ void batch_ensure_device(fv_batch* b, cudaStream_t s) {
     const bool fits =
         b->tiles_ok && fv::tile_smem_bytes(b->f64(), b->t1_cap) <= (size_t)optin;
     b->variant = fits ? fv::kTileVariant : 0;
+    // us per step, shape 0 / 6: FP32 18,056 cells 3.3 / 5.4, 307,332 6.7 / 7.7,
+    // 2,457,668 plain 39.5 / 45.4, compensated 43.7 / 43.2; FP64 70,124 36 / 57,
+    // 307,332 137 / 123 (few large tiles idle most SMs of a small FP64 batch,
+    // while on a large one forming every primitive four times costs more)
+    b->auto_variant = b->f64() && n > 200000 ? b->variant : 0;
   }
 }
 
@@ -1767,8 +1776,8 @@ void build_batch_tiles(fv_batch* b, fv_mesh* const* meshes) {
 }
 
 cudaError_t batch_launch(const fv_batch* b, int mode, const fv::BatchArgs& a, cudaStream_t s) {
-  if (b->variant == 5) return fv::launch_batch_step_tma(b->f64(), mode, a, s);
-  if (b->variant == fv::kTileVariant) return fv::launch_batch_step_tile(b->f64(), mode, a, s);
+  if (b->shape() == 5) return fv::launch_batch_step_tma(b->f64(), mode, a, s);
+  if (b->shape() == fv::kTileVariant) return fv::launch_batch_step_tile(b->f64(), mode, a, s);
   return fv::launch_batch_step(b->f64(), mode, a, b->n_blocks(), s);
 }
 
@@ -1784,6 +1793,7 @@ void batch_enqueue_steps(fv_batch* b, void* U, int64_t j0, int64_t count, double
     a.s.err = b->d_err;
     a.s.wait_limit = fv::kDefaultWaitLimit;
     a.s.drain_limit = fv::kDefaultWaitLimit;
+    a.s.chained = true;
     if (b->use_lo()) {
       a.s.lo = b->d_lo;
       a.s.lo_stage = b->d_lo_stage;
@@ -1800,13 +1810,12 @@ void batch_enqueue_steps(fv_batch* b, void* U, int64_t j0, int64_t count, double
     a.slot_reset = (int)((j + 2) % 3);
     a.t_read = (int)(j % 2);
     a.t_write = (int)((j + 1) % 2);
-    if (b->variant == fv::kTileVariant) {
+    if (b->shape() == fv::kTileVariant) {
       a.s.cell_ln = b->d_cell_ln;
       a.s.tile_info = b->d_tile_info;
       a.s.halo_id = b->d_halo_id;
       a.s.tile = kBatchTile;
       a.s.t1_cap = b->t1_cap;
-      a.s.chained = true;
       a.tile_mesh = b->d_tile_mesh;
       a.tile_start = b->d_tile_start;
       a.tile_cells = b->d_tile_cells;
@@ -1938,6 +1947,7 @@ int fv_batch_set_variant(fv_batch* batch, int32_t variant) {
                 "renumber the meshes with a compact order (Hilbert)");
     }
     batch->variant = variant;
+    batch->shape_chosen = true;
     batch->drop_graph();
   });
 }
@@ -1998,7 +2008,7 @@ int fv_batch_step(fv_batch* batch, void* U, int64_t nsteps, double cfl, double t
       if (chunks > 0) {
         if (!batch->graph || batch->g_U != U || batch->g_scheme != scheme ||
             batch->g_cfl != cfl || batch->g_tstop != t_stop || batch->g_comp != batch->use_lo() ||
-            batch->g_variant != batch->variant) {
+            batch->g_variant != batch->shape()) {
           batch->drop_graph();
           cudaGraph_t g = nullptr;
           FV_CUDA(cudaStreamBeginCapture(batch->cap_stream, cudaStreamCaptureModeThreadLocal));
@@ -2018,7 +2028,7 @@ int fv_batch_step(fv_batch* batch, void* U, int64_t nsteps, double cfl, double t
           batch->g_cfl = cfl;
           batch->g_tstop = t_stop;
           batch->g_comp = batch->use_lo();
-          batch->g_variant = batch->variant;
+          batch->g_variant = batch->shape();
         }
         for (int64_t k = 0; k < chunks; ++k) FV_CUDA(cudaGraphLaunch(batch->graph, s));
       }

@@ -376,6 +376,18 @@ __device__ __forceinline__ void block_dt(const StepArgs& a, double& t, double& d
   }
 }
 
+// The same for mesh m of a batch.
+__device__ __forceinline__ void batch_dt(const BatchArgs& b, int m, double& t, double& dt) {
+  t = b.t[b.t_read * b.n_meshes + m];
+  const unsigned long long bits = b.bmin[b.slot_read * b.n_meshes + m];
+  dt = b.s.cfl > 0.0 ? b.s.cfl * __longlong_as_double((long long)bits) : -b.s.cfl;
+  if (b.s.t_stop > 0.0) {
+    const double rem = b.s.t_stop - t;
+    if (rem < dt) dt = rem;
+    if (!(dt > 0.0)) dt = 0.0;
+  }
+}
+
 // Everything one cell's update reads from its own records.  Geometry layout:
 //   FP64: geom[2i] = (n0x, n0y, n1x, n1y), geom[2i+1] = (n2x, n2y, 1/V, 2V/P),
 //         nbr = int4 (nbr0, nbr1, nbr2, -);

@@ -125,23 +125,6 @@ __global__ void __launch_bounds__(kBlock, var_min_blocks(VAR)) k_step(StepArgs a
 // load_cell / update_cell as the single-mesh kernel, so each mesh advances
 // bit for bit as it would alone.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double batch_step_dt(const BatchArgs& b, int m, double& t) {
-  double dt = 0.0;
-  t = 0.0;
-  if ((threadIdx.x & 31) == 0) {
-    t = b.t[b.t_read * b.n_meshes + m];
-    const unsigned long long bits = b.bmin[b.slot_read * b.n_meshes + m];
-    dt = b.s.cfl > 0.0 ? b.s.cfl * __longlong_as_double((long long)bits) : -b.s.cfl;
-    if (b.s.t_stop > 0.0) {
-      double rem = b.s.t_stop - t;
-      if (rem < dt) dt = rem;
-      if (!(dt > 0.0)) dt = 0.0;
-    }
-  }
-  t = __shfl_sync(0xffffffffu, t, 0);
-  return __shfl_sync(0xffffffffu, dt, 0);
-}
-
 template <typename R, int MODE, bool COMP>
 __global__ void __launch_bounds__(kBlock, sizeof(R) == 4 ? 6 : 1) k_step_batch(BatchArgs b) {
   const StepArgs& a = b.s;
@@ -149,23 +132,28 @@ __global__ void __launch_bounds__(kBlock, sizeof(R) == 4 ? 6 : 1) k_step_batch(B
   const rec_t<R>* __restrict__ geom = static_cast<const rec_t<R>*>(a.geom);
   rec_t<R>* out = static_cast<rec_t<R>*>(a.out);
   const int m = __ldg(b.block_mesh + blockIdx.x);
-  double t = 0.0;
-  const double dt = batch_step_dt(b, m, t);
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;  // cell ids are 32-bit
+  const bool has = i < __ldg(b.mesh_end + m);
+  __shared__ double s_t, s_dt;
+  CellIn<R> c;
+  // as k_step: tables before the grid wait, dt once per block
+  if (has) load_tables<R>(a, geom, i, c);
+  chain_entry();
+  if (has) load_values<R, MODE, COMP>(a, U, i, c);
+  if (threadIdx.x == 0) batch_dt(b, m, s_t, s_dt);
+  R acc[4], perim = R(0);
+  if (has) perim = sum_fluxes<R>(a, U, c, batch_far_field<R>(b, m), acc);
+  __syncthreads();
   R bmin = R(INFINITY);
   bool ok = true;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < __ldg(b.mesh_end + m)) {
-    CellIn<R> cur;
-    load_cell<R, MODE, COMP>(a, U, geom, i, cur);
-    update_cell<R, MODE, COMP>(a, U, out, i, cur, R(dt), batch_far_field<R>(b, m), bmin, ok);
-  }
+  if (has) finish_cell<R, MODE, COMP>(a, out, i, c, acc, perim, R(s_dt), bmin, ok);
   if (MODE == kModeFE || MODE == kModeRK2b) {
     if (!ok) atomicOr(a.err, 1);
     const double mn = (double)block_min<R>(bmin);
     if (threadIdx.x == 0) {
       atomicMin(&b.bmin[b.slot_write * b.n_meshes + m], (unsigned long long)__double_as_longlong(mn));
       if (blockIdx.x == 0 || __ldg(b.block_mesh + blockIdx.x - 1) != m) {  // first block of m
-        b.t[b.t_write * b.n_meshes + m] = t + dt;
+        b.t[b.t_write * b.n_meshes + m] = s_t + s_dt;
         b.bmin[b.slot_reset * b.n_meshes + m] = kInfBits;
       }
     }
@@ -410,12 +398,15 @@ cudaError_t launch_batch_step(bool f64, int mode, const BatchArgs& b, int64_t n_
                               cudaStream_t s) {
   const unsigned g = (unsigned)n_blocks;
   const bool comp = !f64 && b.s.lo != nullptr;
-#define FV_BATCH_CASE(R, C)                                                              \
-  switch (mode) {                                                                        \
-    case kModeFE: k_step_batch<R, kModeFE, C><<<g, kBlock, 0, s>>>(b); break;            \
-    case kModeRK2a: k_step_batch<R, kModeRK2a, C><<<g, kBlock, 0, s>>>(b); break;        \
-    case kModeRK2b: k_step_batch<R, kModeRK2b, C><<<g, kBlock, 0, s>>>(b); break;        \
-    default: return cudaErrorInvalidValue;                                               \
+#define FV_BATCH_CASE(R, C)                                                               \
+  switch (mode) {                                                                         \
+    case kModeFE:                                                                         \
+      return launch_chained(k_step_batch<R, kModeFE, C>, g, kBlock, 0, s, b.s.chained, b); \
+    case kModeRK2a:                                                                       \
+      return launch_chained(k_step_batch<R, kModeRK2a, C>, g, kBlock, 0, s, b.s.chained, b); \
+    case kModeRK2b:                                                                       \
+      return launch_chained(k_step_batch<R, kModeRK2b, C>, g, kBlock, 0, s, b.s.chained, b); \
+    default: return cudaErrorInvalidValue;                                                \
   }
   if (f64) {
     FV_BATCH_CASE(double, false)
@@ -425,7 +416,6 @@ cudaError_t launch_batch_step(bool f64, int mode, const BatchArgs& b, int64_t n_
     FV_BATCH_CASE(float, false)
   }
 #undef FV_BATCH_CASE
-  return cudaGetLastError();
 }
 
 cudaError_t launch_batch_init(unsigned long long* bmin, double* t, int n_meshes, int* err,

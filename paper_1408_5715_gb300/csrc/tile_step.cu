@@ -589,18 +589,7 @@ __global__ void __launch_bounds__(THREADS) k_step_tile_batch(BatchArgs b) {
   const int h1 = __ldg(a.tile_info + 2 * tile + 1);
   chain_entry();
   __shared__ double s_t, s_dt;
-  if (threadIdx.x == 0 && MODE != kModeResidual) {
-    const double t = b.t[b.t_read * b.n_meshes + m];
-    const unsigned long long bits = b.bmin[b.slot_read * b.n_meshes + m];
-    double dt = a.cfl > 0.0 ? a.cfl * __longlong_as_double((long long)bits) : -a.cfl;
-    if (a.t_stop > 0.0) {
-      const double rem = a.t_stop - t;
-      if (rem < dt) dt = rem;
-      if (!(dt > 0.0)) dt = 0.0;
-    }
-    s_t = t;
-    s_dt = dt;
-  }
+  if (threadIdx.x == 0) batch_dt(b, m, s_t, s_dt);
   stage_states<R, THREADS, kStageBatch<R, KMAX>>(U, t0, nt, h1, a.halo_id + hs, sU, sP, a.n,
                                                  a.err);
   __syncthreads();
