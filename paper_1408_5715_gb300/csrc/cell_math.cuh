@@ -268,24 +268,26 @@ __device__ __forceinline__ void face_flux_value(const rec_t<R>& UL, const Prim<R
   X[3] = fma_(na, sub(UR.w, UL.w), add(mul(add(UL.w, L.p), qL), mul(add(UR.w, W.p), qR)));
 }
 
+// first (a constant where it is called): acc starts with this face.
 template <typename R, bool SCALED, int WAVE = kWaveAverage>
 __device__ __forceinline__ void face_flux_acc(const rec_t<R>& UL, const Prim<R>& L,
                                               const rec_t<R>& UR, const Prim<R>& W, R nx, R ny,
-                                              R len, R s, R acc[4]) {
+                                              R len, R s, R acc[4], bool first = false) {
   R X[4];
   face_flux_value<R, SCALED, WAVE>(UL, L, UR, W, nx, ny, len, s, X);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) acc[q] = add(acc[q], X[q]);
+  for (int q = 0; q < 4; ++q) acc[q] = first ? X[q] : add(acc[q], X[q]);
 }
 
 template <typename R, int WAVE = kWaveAverage>
 __device__ __forceinline__ R add_face_flux(const rec_t<R>& UL, const Prim<R>& L, int nb, R nx,
                                            R ny, const rec_t<R>* __restrict__ Ucur,
-                                           const R* uinf, R acc[4], int64_t n, int* err) {
+                                           const R* uinf, R acc[4], int64_t n, int* err,
+                                           bool first = false) {
   const rec_t<R> UR = neighbour_state<R>(UL, nb, nx, ny, Ucur, uinf, n, err);
   const Prim<R> W = primitive<R>(UR);
   const R len = face_len<R>(nx, ny);
-  face_flux_acc<R, false, WAVE>(UL, L, UR, W, nx, ny, len, R(1), acc);
+  face_flux_acc<R, false, WAVE>(UL, L, UR, W, nx, ny, len, R(1), acc, first);
   return len;
 }
 

@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(kBlock) k_step_scaled(StepArgs a, const float*
       const float4 UR = neighbour_state<float>(cur.U, nb[k], nx[k], ny[k], U, a.uinf_f, a.n, a.err);
       const Prim<float> W = primitive<float>(UR);
       const float len = face_len<float>(nx[k], ny[k]);
-      face_flux_acc<float, true>(cur.U, L, UR, W, nx[k], ny[k], len, sc[k], acc);
+      face_flux_acc<float, true>(cur.U, L, UR, W, nx[k], ny[k], len, sc[k], acc, k == 0);
       perim = k == 0 ? len : add(perim, len);
     }
     finish_cell<float, MODE, COMP>(a, out, i, cur, acc, perim, (float)dt, bmin, ok);

@@ -37,8 +37,7 @@ __device__ __forceinline__ R sum_fluxes(const StepArgs& a, const rec_t<R>* __res
                                         const CellIn<R>& c, const R* uinf, R acc[4]) {
   const rec_t<R>& UL = c.U;
   const Prim<R> L = primitive<R>(UL);
-  acc[0] = acc[1] = acc[2] = acc[3] = R(0);
-  R perim = add_face_flux<R, WAVE>(UL, L, c.n0, c.g0.x, c.g0.y, U, uinf, acc, a.n, a.err);
+  R perim = add_face_flux<R, WAVE>(UL, L, c.n0, c.g0.x, c.g0.y, U, uinf, acc, a.n, a.err, true);
   perim = add(perim, add_face_flux<R, WAVE>(UL, L, c.n1, c.g0.z, c.g0.w, U, uinf, acc, a.n, a.err));
   return add(perim,
              add_face_flux<R, WAVE>(UL, L, c.n2, c.g1.x, c.g1.y, U, uinf, acc, a.n, a.err));

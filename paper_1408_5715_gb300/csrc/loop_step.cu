@@ -232,7 +232,6 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
     const float4 UL = src[tid];
     const Prim<float> L = primitive<float>(UL);
     const float nx[3] = {c.g0.x, c.g0.z, c.g1.x}, ny[3] = {c.g0.y, c.g0.w, c.g1.y};
-    acc[0] = acc[1] = acc[2] = acc[3] = 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       float4 UR;
@@ -242,7 +241,7 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
         UR = ghost<float>((int)c.v[k] - 0x10000, UL, nx[k], ny[k], a.uinf);
       const float len = face_len<float>(nx[k], ny[k]);
       face_flux_acc<float, false, WAVE>(UL, L, UR, primitive<float>(UR), nx[k], ny[k], len, 1.f,
-                                        acc);
+                                        acc, k == 0);
       perim = k == 0 ? len : add(perim, len);
     }
   };

@@ -32,7 +32,7 @@ __device__ __forceinline__ Prim<R> rec_prim(const rec_t<R>& p) {
 template <typename R, int WAVE = kWaveAverage, bool PRIMS = true>
 __device__ __forceinline__ R smem_face(const rec_t<R>& UL, const Prim<R>& L, unsigned v, R nx, R ny,
                                        const rec_t<R>* sU, const rec_t<R>* sP, const R* uinf,
-                                       R acc[4], int cap, int* err) {
+                                       R acc[4], int cap, int* err, bool first = false) {
   rec_t<R> UR;
   Prim<R> W;
   if (v < kGhostCodes) {
@@ -48,7 +48,7 @@ __device__ __forceinline__ R smem_face(const rec_t<R>& UL, const Prim<R>& L, uns
     W = primitive<R>(UR);
   }
   const R len = face_len<R>(nx, ny);
-  face_flux_acc<R, false, WAVE>(UL, L, UR, W, nx, ny, len, R(1), acc);
+  face_flux_acc<R, false, WAVE>(UL, L, UR, W, nx, ny, len, R(1), acc, first);
   return len;
 }
 
@@ -60,7 +60,7 @@ __device__ __forceinline__ R cell_fluxes(const rec_t<R>& g0, const rec_t<R>& g1,
                                          const rec_t<R>* sP, const R* uinf, R acc[4], int cap,
                                          int* err) {
   R perim = smem_face<R, WAVE, PRIMS>(UL, L, ln.x & 0xffffu, g0.x, g0.y, sU, sP, uinf, acc, cap,
-                                      err);
+                                      err, true);
   perim = add(perim, smem_face<R, WAVE, PRIMS>(UL, L, ln.x >> 16, g0.z, g0.w, sU, sP, uinf, acc,
                                                cap, err));
   // the high half of ln.y holds a node id in the vertex-geometry layout

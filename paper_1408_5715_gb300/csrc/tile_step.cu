@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(THREADS + 32) k_step_faces64(StepArgs a) {
       const int i = t0 + e;
       dq4 base{};
       if (MODE == kModeRK2b) base = static_cast<const dq4*>(a.Ubase)[i];
-      // (the other shapes start from zero: the same up to the sign of a zero)
+      // the faces in order, as every shape adds them
       auto flux = [&](unsigned r) {  // bit 15: the face was evaluated from the other side
         const unsigned at = r & 0x7fffu, sign = (r & 0x8000u) << 16;
         const dq4 x = get(sF, index_ok(at, a.f_cap, a.err) ? at : 0u);

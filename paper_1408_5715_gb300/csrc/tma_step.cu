@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kBlock) k_step_tma(BatchArgs b) {
         }
         const Prim<R> W = primitive<R>(UR);
         const R len = face_len<R>(nx[q], ny[q]);
-        face_flux_acc<R, false>(c.U, L, UR, W, nx[q], ny[q], len, R(1), acc);
+        face_flux_acc<R, false>(c.U, L, UR, W, nx[q], ny[q], len, R(1), acc, q == 0);
         perim = q == 0 ? len : add(perim, len);
       }
       finish_cell<R, MODE, COMP>(a, out, i, c, acc, perim, dtR, bmin, ok);
