@@ -568,6 +568,7 @@ void ensure_device(fv_mesh* m, cudaStream_t s) {
       FV_CUDA(cudaMalloc((void**)&m->d_lo_stage, nn * sizeof(uint2)));
     }
     FV_CUDA(cudaMalloc((void**)&m->d_scal, sizeof(fv::LoopScalars)));
+    FV_CUDA(fv::launch_init_aux(m->d_scal, s));
     FV_CUDA(cudaMalloc((void**)&m->d_partials, fv::kTotalsBlocks * 4 * sizeof(double)));
     FV_CUDA(cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking));
     m->dev_n = n;
@@ -1505,14 +1506,11 @@ int fv_compute_dt(fv_mesh* mesh, const void* U, double cfl, void* stream, double
     cudaStream_t s = as_stream(stream);
     ensure_device(mesh, s);
     fv::LoopScalars* sc = mesh->d_scal;
-    FV_CUDA(fv::launch_reset_min(&sc->aux_bmin, &sc->aux_err, s));
-    FV_CUDA(fv::launch_bound(mesh->f64(), U, mesh->d_geom, mesh->h.n, &sc->aux_bmin, &sc->aux_err,
-                             s));
-    FV_CUDA(fv::launch_dt_from_bound(&sc->aux_bmin, cfl, &sc->dt_out, s));
+    FV_CUDA(fv::launch_compute_dt(mesh->f64(), U, mesh->d_geom, mesh->h.n, cfl, sc, s));
     fv::LoopScalars h{};
     FV_CUDA(cudaMemcpyAsync(&h, sc, sizeof h, cudaMemcpyDeviceToHost, s));
     FV_CUDA(cudaStreamSynchronize(s));
-    if (h.aux_err) throw fv::Error{FV_ENONFINITE, "state has non-finite values or rho/p <= 0"};
+    if (h.dt_err) throw fv::Error{FV_ENONFINITE, "state has non-finite values or rho/p <= 0"};
     *dt = h.dt_out;
   });
 }
@@ -1530,7 +1528,7 @@ int fv_conserved_totals(fv_mesh* mesh, const void* U, double* out, void* stream)
     ensure_device(mesh, s);
     fv::LoopScalars* sc = mesh->d_scal;
     FV_CUDA(fv::launch_totals(mesh->f64(), U, mesh->d_vol, mesh->h.n, mesh->d_partials,
-                              sc->totals, s));
+                              &sc->totals_ticket, sc->totals, s));
     FV_CUDA(cudaMemcpyAsync(out, sc->totals, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
     FV_CUDA(cudaStreamSynchronize(s));
   });

@@ -259,24 +259,70 @@ __global__ void __launch_bounds__(kBlock) k_bound(const rec_t<R>* __restrict__ U
   if (threadIdx.x == 0) atomicMin(bmin, (unsigned long long)__double_as_longlong(m));
 }
 
-__global__ void k_set_u64(unsigned long long* p, unsigned long long v, int* flag) {
-  *p = v;
-  if (flag) *flag = 0;
-}
-
-__global__ void k_dt_from_bound(const unsigned long long* bmin, double cfl, double* dt) {
-  *dt = cfl > 0.0 ? cfl * __longlong_as_double((long long)*bmin) : -cfl;
-}
-
-// Deterministic totals sum_T V_T U_T in FP64: a fixed grid, a fixed
-// thread-to-cell assignment and fixed reduction trees.
+// fv_compute_dt in one launch: the blocks' minima and error meet in the aux
+// scalars (at rest +inf and 0), the last block to finish forms dt and puts the
+// scalars back.
 template <typename R>
-__global__ void __launch_bounds__(kBlock) k_totals_partial(const rec_t<R>* __restrict__ U,
-                                                           const double* __restrict__ vol,
-                                                           int64_t n, double* partials) {
+__global__ void __launch_bounds__(kBlock) k_compute_dt(const rec_t<R>* __restrict__ U,
+                                                       const rec_t<R>* __restrict__ geom, int64_t n,
+                                                       double cfl, LoopScalars* sc) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  R b = R(INFINITY);
+  bool ok = true;
+  if (i < n) b = cell_bound<R>(Rec<R>::ld(U + i), geom_inradius<R>(geom, i), ok);
+  const bool bad = __syncthreads_or(!ok);
+  const R m = block_min<R>(b);
+  if (threadIdx.x != 0) return;
+  if (bad) atomicOr(&sc->aux_err, 1);
+  atomicMin(&sc->aux_bmin, (unsigned long long)__double_as_longlong((double)m));
+  __threadfence();
+  if (atomicInc(&sc->aux_ticket, gridDim.x - 1) != gridDim.x - 1) return;
+  __threadfence();
+  const unsigned long long bits = atomicExch(&sc->aux_bmin, kInfBits);
+  sc->dt_out = cfl * __longlong_as_double((long long)bits);
+  sc->dt_err = atomicExch(&sc->aux_err, 0);
+}
+
+__global__ void k_init_aux(LoopScalars* sc) {
+  sc->aux_bmin = kInfBits;
+  sc->aux_err = sc->dt_err = 0;
+  sc->aux_ticket = sc->totals_ticket = 0u;
+}
+
+// Deterministic totals sum_T V_T U_T in FP64: a thread-to-cell assignment
+// fixed by the number of cells (kTotalsBlocks blocks at most) and fixed
+// reduction trees; the last block to finish adds the partials, in block order.
+// Warps without cells leave the tree out (their sums are zero): on 41,410
+// cells, seven of eight warps of the full grid, whose additions alone held the
+// FP64 pipe for some 10 us.
+template <typename R>
+__global__ void __launch_bounds__(kBlock) k_totals(const rec_t<R>* __restrict__ U,
+                                                   const double* __restrict__ vol, int64_t n,
+                                                   double* partials, unsigned* ticket,
+                                                   double* out) {
+  __shared__ double sm[4][kBlock / 32];
+  __shared__ bool last;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double s[4] = {0.0, 0.0, 0.0, 0.0};
+  auto block_sum = [&](bool any, double* to) {  // any: uniform in the warp
+    if (any) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+    }
+    if (lane == 0)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sm[q][warp] = s[q];
+    __syncthreads();
+    if (threadIdx.x < 4) {
+      double acc = 0.0;
+      for (int w = 0; w < kBlock / 32; ++w) acc += sm[threadIdx.x][w];
+      to[threadIdx.x] = acc;
+    }
+  };
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+  const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int64_t i = first; i < n; i += stride) {
     const rec_t<R> u = Rec<R>::ld(U + i);
     const double v = __ldg(vol + i);
     s[0] += v * (double)u.x;
@@ -284,40 +330,18 @@ __global__ void __launch_bounds__(kBlock) k_totals_partial(const rec_t<R>* __res
     s[2] += v * (double)u.z;
     s[3] += v * (double)u.w;
   }
-  __shared__ double sm[4][kBlock / 32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
-    if (lane == 0) sm[q][warp] = s[q];
-  }
+  block_sum(first - lane < n, partials + 4 * blockIdx.x);
+  if (threadIdx.x < 4) __threadfence();
   __syncthreads();
-  if (threadIdx.x < 4) {
-    double acc = 0.0;
-    for (int w = 0; w < kBlock / 32; ++w) acc += sm[threadIdx.x][w];
-    partials[4 * blockIdx.x + threadIdx.x] = acc;
-  }
-}
-
-__global__ void __launch_bounds__(kBlock) k_totals_final(const double* partials, int nparts,
-                                                         double* out) {
-  double s[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int j = threadIdx.x; j < nparts; j += blockDim.x)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) s[q] += partials[4 * j + q];
-  __shared__ double sm[4][kBlock / 32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
-    if (lane == 0) sm[q][warp] = s[q];
-  }
+  if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
   __syncthreads();
-  if (threadIdx.x < 4) {
-    double acc = 0.0;
-    for (int w = 0; w < kBlock / 32; ++w) acc += sm[threadIdx.x][w];
-    out[threadIdx.x] = acc;
-  }
+  if (!last) return;
+  __threadfence();
+  s[0] = s[1] = s[2] = s[3] = 0.0;
+  for (int j = threadIdx.x; j < (int)gridDim.x; j += blockDim.x)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s[q] += __ldcg(partials + 4 * j + q);
+  block_sum((threadIdx.x & ~31u) < gridDim.x, out);
 }
 
 inline unsigned grid_for(int64_t n) { return (unsigned)((n + kBlock - 1) / kBlock); }
@@ -469,14 +493,14 @@ cudaError_t launch_bound(bool f64, const void* U, const void* geom, int64_t n,
 }
 
 cudaError_t launch_totals(bool f64, const void* U, const double* vol, int64_t n, double* partials,
-                          double* out, cudaStream_t s) {
+                          unsigned* ticket, double* out, cudaStream_t s) {
+  const int64_t want = (n + kBlock - 1) / kBlock;
+  const unsigned g = (unsigned)(want < 1 ? 1 : want > kTotalsBlocks ? kTotalsBlocks : want);
   if (f64)
-    k_totals_partial<double><<<kTotalsBlocks, kBlock, 0, s>>>(static_cast<const dq4*>(U), vol, n,
-                                                              partials);
+    k_totals<double><<<g, kBlock, 0, s>>>(static_cast<const dq4*>(U), vol, n, partials, ticket, out);
   else
-    k_totals_partial<float><<<kTotalsBlocks, kBlock, 0, s>>>(static_cast<const float4*>(U), vol,
-                                                             n, partials);
-  k_totals_final<<<1, kBlock, 0, s>>>(partials, kTotalsBlocks, out);
+    k_totals<float><<<g, kBlock, 0, s>>>(static_cast<const float4*>(U), vol, n, partials, ticket,
+                                         out);
   return cudaGetLastError();
 }
 
@@ -562,14 +586,20 @@ cudaError_t launch_restrict_mean(bool fine_f64, bool coarse_f64, const void* Uf,
   return cudaGetLastError();
 }
 
-cudaError_t launch_reset_min(unsigned long long* bmin, int* flag, cudaStream_t s) {
-  k_set_u64<<<1, 1, 0, s>>>(bmin, kInfBits, flag);
+cudaError_t launch_init_aux(LoopScalars* sc, cudaStream_t s) {
+  k_init_aux<<<1, 1, 0, s>>>(sc);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dt_from_bound(const unsigned long long* bmin, double cfl, double* dt_out,
-                                 cudaStream_t s) {
-  k_dt_from_bound<<<1, 1, 0, s>>>(bmin, cfl, dt_out);
+cudaError_t launch_compute_dt(bool f64, const void* U, const void* geom, int64_t n, double cfl,
+                              LoopScalars* sc, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  if (f64)
+    k_compute_dt<double><<<grid_for(n), kBlock, 0, s>>>(
+        static_cast<const dq4*>(U), static_cast<const dq4*>(geom), n, cfl, sc);
+  else
+    k_compute_dt<float><<<grid_for(n), kBlock, 0, s>>>(
+        static_cast<const float4*>(U), static_cast<const float4*>(geom), n, cfl, sc);
   return cudaGetLastError();
 }
 

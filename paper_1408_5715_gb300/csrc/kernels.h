@@ -9,7 +9,7 @@
 namespace fv {
 
 constexpr int kBlock = 256;        // threads per block of the cell kernels
-constexpr int kTotalsBlocks = 1024; // fixed grid of the deterministic totals
+constexpr int kTotalsBlocks = 1024; // largest grid of the deterministic totals
 
 // Wave speed of the Lax-Friedrichs dissipation (StepArgs::wave).
 constexpr int kWaveAverage = 0;  // interface averages (Sec. 6.2.2, the default)
@@ -34,9 +34,11 @@ struct LoopScalars {
   int pad;
   double totals[4];
   double dt_out;
-  unsigned long long aux_bmin;  // minimum of fv_compute_dt, apart from the loop's
-  int aux_err;
-  int pad2;
+  // fv_compute_dt and fv_conserved_totals, apart from the loop: at rest +inf
+  // and zeros (the last block of each call puts them back)
+  unsigned long long aux_bmin;
+  int aux_err, dt_err;
+  unsigned aux_ticket, totals_ticket;
 };
 
 // Arguments of the fused step kernel (precision-independent view; the
@@ -309,8 +311,8 @@ cudaError_t launch_init_scalars(LoopScalars* d, cudaStream_t s);
 cudaError_t launch_bound(bool f64, const void* U, const void* geom, int64_t n,
                          unsigned long long* bmin, int* err, cudaStream_t s);
 cudaError_t launch_totals(bool f64, const void* U, const double* vol, int64_t n,
-                          double* partials /*[kTotalsBlocks*4]*/, double* out /*[4]*/,
-                          cudaStream_t s);
+                          double* partials /*[kTotalsBlocks*4]*/, unsigned* ticket /*0*/,
+                          double* out /*[4]*/, cudaStream_t s);
 cudaError_t launch_batch_step(bool f64, int mode, const BatchArgs& b, int64_t n_blocks,
                               cudaStream_t s);
 cudaError_t launch_batch_init(unsigned long long* bmin, double* t, int n_meshes, int* err,
@@ -322,9 +324,9 @@ cudaError_t launch_batch_totals(bool f64, const void* U, const double* vol, cons
                                 const int64_t* mesh_end, const int* mesh_first_block,
                                 int n_meshes, int64_t n_blocks, double* partials, double* out,
                                 cudaStream_t s);
-// *bmin = +inf bits, *flag = 0 (flag nullable)
-cudaError_t launch_reset_min(unsigned long long* bmin, int* flag, cudaStream_t s);
-cudaError_t launch_dt_from_bound(const unsigned long long* bmin, double cfl, double* dt_out,
-                                 cudaStream_t s);
+// the aux scalars at rest; dt of fv_compute_dt (cfl > 0) into sc->dt_out, dt_err
+cudaError_t launch_init_aux(LoopScalars* sc, cudaStream_t s);
+cudaError_t launch_compute_dt(bool f64, const void* U, const void* geom, int64_t n, double cfl,
+                              LoopScalars* sc, cudaStream_t s);
 
 }  // namespace fv
