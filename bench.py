@@ -130,7 +130,8 @@ def measured_peaks():
 
 
 KERNEL_SOURCES = ("kernels.h", "cell_math.cuh", "tile_math.cuh", "tma_util.cuh",
-                  "launch_util.cuh", "kernels.cu", "tile_step.cu", "tma_step.cu", "pair_step.cu")
+                  "launch_util.cuh", "kernels.cu", "tile_step.cu", "tma_step.cu", "pair_step.cu",
+                  "loop_step.cu")
 
 
 def kernel_source_hash():
@@ -357,7 +358,8 @@ def run_ours(args):
                     "k_face_scales" + ("_tc" if args.closure_engine == "tcgen05" else "")
                     + " + k_step_scaled")
         else:
-            kfun = {5: "k_step_tma", 6: "k_step_tile", 7: "k_step_tile_faces"}.get(
+            kfun = {5: "k_step_tma", 6: "k_step_tile",
+                    7: "k_step_faces64" if prec == "f64" else "k_step_tile_faces"}.get(
                 tune["variant"], "k_step")
         kname = (f"{kfun}<{'float' if prec == 'f32' else 'double'}, "
                  f"{'RK2' if stages == 2 else 'FE'}, "
@@ -406,7 +408,7 @@ def run_ours(args):
                          else f"step_{prec}{'' if comp or prec == 'f64' else '_plain'}"
                               f"_{args.workload}.md")},
         "e2e": e2e,
-        "gpu_launches": args.steps * (launches + 4),
+        "gpu_launches": args.steps * (launches + 3),
         "clocks": clk.summary(),
     }
     if rank == 0 and not args.no_extras and world == 1:
