@@ -466,6 +466,20 @@ size_t pair_smem(const fv_mesh* m) {
   return fv::pair_smem_bytes(m->p_e_cap, m->p_t1_cap, m->tiles_built, m->pair_staged != 0);
 }
 
+// Builds tables that a quicker default path wants; false where they do not fit
+// (in the tiles' limits or in memory), and the call takes the path without them.
+template <typename F>
+bool optional_tables(F&& build) {
+  try {
+    build();
+    return true;
+  } catch (const fv::Error&) {
+  } catch (const std::bad_alloc&) {
+  }
+  cudaGetLastError();
+  return false;
+}
+
 // Tiles of the resident loop for a small FP32 mesh, up to kLoopMaxTiles of
 // them; other meshes run a launch per step.
 void build_loop(fv_mesh* m, cudaStream_t s) {
@@ -523,14 +537,10 @@ void choose_shape(fv_mesh* m, cudaStream_t s) {
   if (tiled) {
     m->auto_variant = m->f64() ? fv::kFaceTileVariant : fv::kTileVariant;
     m->auto_tile = (int)(m->f64() ? fp64_tile(n) : quick_tile(n));
-    bool good = true;
-    try {
+    bool good = optional_tables([&] {
       ensure_tiles(m, s);
       check_tile_smem(m, step_tile_smem(m));
-    } catch (const fv::Error& e) {
-      if (e.code != FV_EINVAL) throw;
-      good = false;
-    }
+    });
     good = good && (m->f64() ? 2 * m->tiles_halo_cells <= 5 * n
                              : m->tiles_quick && 4 * m->tiles_halo_cells <= 3 * n);
     if (good) return;
@@ -583,7 +593,7 @@ void ensure_device(fv_mesh* m, cudaStream_t s) {
     FV_CUDA(cudaMemcpyAsync(m->d_vol, m->h.vol.data(), n * sizeof(double), cudaMemcpyHostToDevice,
                             s));
     FV_CUDA(cudaStreamSynchronize(s));  // lay is a local staging buffer
-    build_loop(m, s);
+    if (!optional_tables([&] { build_loop(m, s); })) m->free_loop();
   }
   FV_CUDA(cudaStreamSynchronize(s));
   m->device = dev;
