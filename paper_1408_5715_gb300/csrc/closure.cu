@@ -307,6 +307,9 @@ __device__ __forceinline__ void load_face(const StepArgs& a, const FaceRec* face
 __global__ void __launch_bounds__(kClThreads) k_face_scales(StepArgs a, const FaceRec* faces,
                                                             int64_t nf, ClosureParams cp,
                                                             float* s_cf) {
+  // waiting before the weights are read, not after: 6,720 cells, both passes,
+  // 6.9 -> 5.95 us per step; 250,000 cells 14.35 -> 14.2
+  chain_entry();
   __shared__ ClShared sh;
   load_small_params(cp, sh);
   ClFrag fr;
@@ -315,7 +318,6 @@ __global__ void __launch_bounds__(kClThreads) k_face_scales(StepArgs a, const Fa
   ClWarpSmem& w = sh.warp[warp];
   const int64_t wstride = (int64_t)gridDim.x * kClWarps * 32;
   int64_t row = ((int64_t)blockIdx.x * kClWarps + warp) * 32 + lane;
-  chain_entry();
   // this round's face and, issued before this round computes, the next's
   FaceIn cur, nxt;
   for (int64_t base = row - lane; base < nf; base += wstride, row += wstride) {
