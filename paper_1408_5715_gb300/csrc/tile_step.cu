@@ -351,12 +351,15 @@ __device__ __forceinline__ bool rough_bound(const dq4& U, double inradius, float
               E = rough_float(U.w, big), r = rough_float(inradius, big);
   const float ir = recip<float>(rho), u = mx * ir, v = my * ir;
   const float pe = E - 0.5f * (mx * u + my * v);  // p / (gamma - 1)
-  b = r * recip<float>(root<float>(u * u + v * v) +
-                       root<float>((float)(kGamma * kGammaM1) * pe * ir));
+  const float vv = u * u + v * v, cc = (float)(kGamma * kGammaM1) * pe * ir;
+  b = r * recip<float>(root<float>(vv) + root<float>(cc));
   // rounding moves pe by at most a few 2^-23 E: at pe > E / 100 the sound
-  // speed is good to 4e-5, and the exact pressure is positive too
+  // speed is good to 4e-5, and the exact pressure is positive too.  The squares
+  // and the bound have limits of their own: speeds of ordinary rho and pe can
+  // leave the floats' range (then b would be 0 or infinite), and at cc > 1e-24
+  // what vv loses below the normal floats is nothing beside c
   return !big && rho > 1e-20f && rho < 1e20f && E < 1e20f && pe > 0.01f * E && pe > 1e-20f &&
-         r > 1e-20f;
+         r > 1e-20f && vv < 1e30f && cc > 1e-24f && cc < 1e30f && b < 1e38f;
 }
 
 // Shape 7 in FP64, bound by the FP64 pipe (two lanes a clock and SM): 84 % of
