@@ -509,7 +509,8 @@ cudaError_t launch_totals(bool f64, const void* U, const double* vol, int64_t n,
 // FP64 in the order j = 0, 1, ... and written in the coarse precision.
 // Bound by the FP64 pipe (five operations a child, 19 clocks each per warp and
 // SM).  A float result takes one reciprocal and four products instead of four
-// divisions (within 2 ulp of FP64, before its rounding to float), and VEC
+// divisions (within 2 ulp of FP64, before its rounding to float) where the area
+// sum is in [2^-100, 2^100), and VEC
 // reads the ids four at a time (kids a multiple of 4, fine_of 16-byte
 // aligned), so that four children's states are on their way together.
 // 250,000 cells of 16 FP64 children: 87 -> 77 us a call.
@@ -553,7 +554,8 @@ __global__ void __launch_bounds__(kBlock) k_restrict_mean(const rec_t<RF>* __res
       m.add_child(Rec<RF>::ld(Uf + f), __ldg(area + f));
     }
   }
-  if constexpr (sizeof(RC) == 4) {
+  // the reciprocal of a tiny area sum would overflow where the means do not
+  if (sizeof(RC) == 4 && in_quick_range(m.v)) {
     const double r = recip<double>(m.v);
     Uc[c] = Rec<RC>::make((RC)(m.s[0] * r), (RC)(m.s[1] * r), (RC)(m.s[2] * r), (RC)(m.s[3] * r));
   } else {
