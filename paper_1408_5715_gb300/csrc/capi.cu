@@ -96,9 +96,13 @@ struct fv_closure {
   // with another closure at the same address is recaptured
   uint64_t version = 0;
   // training scratch: per-cell terms, per-block gradient and loss partials
-  // (scratch.cells grows to the largest mesh trained on)
+  // (scratch.cells grows to the largest mesh trained on).  An array that a call
+  // in the caller's stream capture used is kept until the closure goes: the
+  // caller's graph may be replayed after the array was outgrown.
   fv::ClosureScratch scratch{};
   int64_t cells_cap = 0;
+  bool cells_captured = false;
+  std::vector<float4*> cells_outgrown;
   float* d_grad = nullptr;
 
   fv::ClosureParams params() const {
@@ -277,6 +281,17 @@ namespace {
 // numbering and tile size and copied to the device.
 bool tiled_shape(int v) { return v == fv::kTileVariant || v == fv::kFaceTileVariant; }
 bool uses_tiles(const fv_mesh* m) { return m->blocking == 2 || tiled_shape(m->shape()); }
+
+// Whether the caller captures stream s into a graph (of its own): the call
+// must not synchronise, and what it launches may be replayed at any later time.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside another stream's capture
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
 
 // Several host arrays for one device allocation and one copy.
 struct Staging {
@@ -2114,6 +2129,29 @@ void check_closure(const fv_closure* c) {
   if (!c) invalid("null closure");
 }
 
+// Per-cell terms of the training kernels for a mesh of n cells.
+void ensure_grad_cells(fv_closure* c, int64_t n, cudaStream_t s) {
+  const bool captured = capturing(s);
+  if (c->cells_cap < n) {
+    if (c->scratch.cells && (captured || c->cells_captured)) {
+      c->cells_outgrown.push_back(c->scratch.cells);
+      c->scratch.cells = nullptr;
+    }
+    // the stream may still read the smaller array (cudaFree waits for it)
+    dev_free(c->scratch.cells);
+    c->cells_cap = 0;
+    c->cells_captured = false;
+    // an allocation is no part of a capture, but this thread may be barred from it meanwhile
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (captured) FV_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = cudaMalloc((void**)&c->scratch.cells, n * sizeof(float4));
+    if (captured) cudaThreadExchangeStreamCaptureMode(&mode);
+    FV_CUDA(e);
+    c->cells_cap = n;
+  }
+  c->cells_captured = c->cells_captured || captured;
+}
+
 }  // namespace
 
 extern "C" {
@@ -2163,6 +2201,7 @@ int fv_closure_destroy(fv_closure* closure) {
     cudaFree(closure->d_b);
     cudaFree(closure->d_theta);
     cudaFree(closure->scratch.cells);
+    for (float4* p : closure->cells_outgrown) cudaFree(p);
     cudaFree(closure->scratch.gpart);
     cudaFree(closure->scratch.lpart);
     cudaFree(closure->d_grad);
@@ -2224,13 +2263,7 @@ int fv_closure_loss_grad(fv_mesh* mesh, const void* U0, const void* Ut, double d
     ensure_device(mesh, s);
     fv::StepArgs a = base_args(mesh);
     a.U = U0;
-    if (closure->cells_cap < mesh->h.n) {
-      // the stream may still read the smaller array (cudaFree waits for it)
-      dev_free(closure->scratch.cells);
-      closure->cells_cap = 0;
-      FV_CUDA(cudaMalloc((void**)&closure->scratch.cells, mesh->h.n * sizeof(float4)));
-      closure->cells_cap = mesh->h.n;
-    }
+    ensure_grad_cells(closure, mesh->h.n, s);
     FV_CUDA(fv::launch_closure_grad(a, static_cast<const float*>(Ut), dt, weights,
                                     closure->params(), closure->scratch,
                                     grad ? grad : closure->d_grad, s));
