@@ -135,6 +135,9 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int k = tid; k < 2 * kRow; k += THREADS + 32) (&s_min[0][0])[k] = INFINITY;
+  // read here: block 0 may write the time at the end of a launch of one bound
+  // before another block's warp of dt has begun
+  double t = warp == kWarps ? *a.t : 0.0;
   cluster_sync();  // every block's mbarriers are ready
 
   if (warp == kWarps) {
@@ -145,7 +148,7 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
       mbar_expect_tx(&min_bar[0], min_bytes);
       mbar_expect_tx(&min_bar[1], min_bytes);
     }
-    double t = *a.t, dt_raw = 0.0;
+    double dt_raw = 0.0;
     unsigned epoch = 0u, minima = 0u;
     // a ring's epoch is over: its mbarrier is armed for the one after next
     auto rearm_ring = [&]() {
