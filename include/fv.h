@@ -221,10 +221,11 @@ int fv_mesh_autotune(fv_mesh* mesh, const void* U, int32_t scheme, void* stream,
                      double* us_per_step);
 
 /* Polls of a device-side wait before it gives up (shape 5 waits for its bulk
- * copies on mbarriers).  A wait that gives up makes the kernel stop, drain its
- * own copies in flight (with the default limit) and set an error bit, and
- * fv_step / fv_mesh_status return FV_ETIMEOUT; the state is then not valid.
- * If the drain gives up as well they return FV_ESTATE.
+ * copies on mbarriers, the resident loop of small meshes for what its blocks
+ * send each other, there 2^20 times at most).  A wait that gives up makes the
+ * kernel stop, drain its own copies in flight (with the default limit) and set
+ * an error bit, and fv_step / fv_mesh_status return FV_ETIMEOUT; the state is
+ * then not valid.  If the drain gives up as well they return FV_ESTATE.
  * Default 2^24.  A limit of 0 forces the timeout path (for tests). */
 int fv_mesh_set_wait_limit(fv_mesh* mesh, uint32_t polls);
 

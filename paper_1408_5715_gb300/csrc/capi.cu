@@ -192,7 +192,7 @@ struct fv_mesh {
   int* loop_ring = nullptr;       // cells of the tiles' rings
   unsigned* loop_push = nullptr;  // where the tiles' edge cells go
   bool pair_default = true;  // fv_mesh_set_blocking left the tile size to the library
-  unsigned wait_limit = fv::kDefaultWaitLimit;  // bounded device waits (variant 5)
+  unsigned wait_limit = fv::kDefaultWaitLimit;  // bounded device waits (variant 5, resident loop)
   fv::LoopScalars* d_scal = nullptr;
   double* d_partials = nullptr;
   cudaStream_t cap_stream = nullptr;
@@ -859,7 +859,8 @@ void enqueue_loop(fv_mesh* m, void* U, int64_t nsteps, double cfl, double t_stop
   a.t_stop = t_stop;
   a.fixed_dt = !(cfl > 0.0);
   a.clamp = t_stop > 0.0;
-  a.polls = kLoopPolls;
+  a.polls = std::min(m->wait_limit, kLoopPolls);
+  a.drain_polls = kLoopPolls;
   a.steps_per_bound = m->blocking;
   a.t = &m->d_scal->t[0];
   a.err = &m->d_scal->err;

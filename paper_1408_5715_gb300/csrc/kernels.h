@@ -288,6 +288,7 @@ struct LoopArgs {
   double cfl, t_stop;         // as StepArgs; with fixed_dt (cfl < 0), clamp (t_stop > 0)
   bool fixed_dt, clamp;
   unsigned polls;             // tries of a wait before it gives up (error bit 2)
+  unsigned drain_polls;       // ... for the stores on their way to a block that gave up (bit 4)
   int nsteps;
   int steps_per_bound;        // 1, or 2: two steps share one CFL bound
   double* t;                  // time advanced, read and written

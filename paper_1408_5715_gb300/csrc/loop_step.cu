@@ -20,8 +20,14 @@
 // Each mbarrier has a twin: stages of even and odd number (epoch) use their
 // own, so what a quick neighbour sends ahead never counts for the stage still
 // awaited; it cannot be two stages ahead, since its stage needs this block's
-// last one.  Waits are bounded: one that gives up sets error bit 2, and the
-// blocks that wait for it give up in turn.
+// last one.
+//
+// Waits are bounded.  A block in which one gives up (error bit 2) stops as a
+// whole at the barrier that follows every wait, so it has pushed its stages
+// whole or not at all, and the blocks that wait for it give up in turn.  Every
+// block leaves the number of stages it pushed with all others before the
+// closing cluster barrier; one that gave up then knows which stores are still
+// on their way to it and awaits those (drain) before it leaves.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -61,6 +67,16 @@ __device__ __forceinline__ void push_value(unsigned to, float v, unsigned bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(
                    to),
                "f"(v), "r"(bar)
+               : "memory");
+}
+
+__device__ __forceinline__ void store_remote(unsigned to, unsigned x, unsigned y) {
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(to), "r"(x), "r"(y) : "memory");
+}
+// Takes bytes that will not come off what an mbarrier of this block expects.
+__device__ __forceinline__ void forgo_tx(uint64_t* bar, unsigned bytes) {
+  asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)),
+               "r"(bytes)
                : "memory");
 }
 
@@ -118,6 +134,8 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
   __shared__ __align__(16) float s_min[2][kRow];
   __shared__ float s_dt;
   __shared__ __align__(8) uint64_t ring_bar[2], min_bar[2];  // of even and odd epochs
+  // by block: the last ring epoch and the number of minima it has pushed
+  __shared__ uint2 s_sent[kLoopMaxTiles];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = blockIdx.x, blocks = gridDim.x;  // the grid is one cluster
   const int4 info = __ldg(a.info + rank);           // ring offset, ring size, edge cells, pushes
@@ -141,7 +159,9 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
   cluster_sync();  // every block's mbarriers are ready
 
   if (warp == kWarps) {
-    // ring epochs 1, 2, ... (states after each stage), minima 0, 1, ...
+    // ring epochs 1, 2, ... (states after each stage), minima 0, 1, ...; of
+    // each kind the last two armed may be under way
+    unsigned armed_ring = 2u, armed_min = 1u;
     if (lane == 0) {
       mbar_expect_tx(&ring_bar[1], ring_bytes);
       mbar_expect_tx(&ring_bar[0], ring_bytes);
@@ -150,18 +170,22 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
     }
     double dt_raw = 0.0;
     unsigned epoch = 0u, minima = 0u;
-    // a ring's epoch is over: its mbarrier is armed for the one after next
+    // every compute thread has awaited this epoch's ring (they passed the
+    // barrier after that wait): its mbarrier is armed for the one after next
     auto rearm_ring = [&]() {
-      if (!await(&ring_bar[epoch & 1u], ((epoch - 1u) >> 1) & 1u, fail ? 0u : a.polls))
-        fail = true;
       if (lane == 0) mbar_expect_tx(&ring_bar[epoch & 1u], ring_bytes);
+      armed_ring = epoch + 2u;
     };
     bool due = true;
     for (int j = 0; j < a.nsteps; ++j) {
       if (due) {
         const unsigned p = minima & 1u;
-        if (!await(&min_bar[p], (minima >> 1) & 1u, fail ? 0u : a.polls)) fail = true;
-        if (lane == 0) mbar_expect_tx(&min_bar[p], min_bytes);
+        if (__all_sync(0xffffffffu, await(&min_bar[p], (minima >> 1) & 1u, a.polls))) {
+          armed_min = minima + 2u;
+          if (lane == 0) mbar_expect_tx(&min_bar[p], min_bytes);
+        } else {
+          fail = true;
+        }
         float m = INFINITY;
 #pragma unroll
         for (int k = 0; k < kRow / 128; ++k) {
@@ -185,16 +209,38 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
       due = a.steps_per_bound == 1 || !due;
       if (epoch > 0u) rearm_ring();  // the ring this step reads
       ++epoch;
-      if (RK2) __syncthreads();  // B
-      if (j + 1 == a.nsteps) break;
-      __syncthreads();  // A
       if (RK2) {
-        rearm_ring();  // U*'s, which every thread has awaited by now
+        if (__syncthreads_or(fail)) break;  // B: U*'s ring was awaited
+        rearm_ring();
         ++epoch;
       }
+      if (j + 1 == a.nsteps) break;
+      __syncthreads();  // A
     }
-    if (!__syncthreads_or(fail) && rank == 0 && lane == 0) *a.t = t;
-    cluster_sync();
+    const bool failed = __syncthreads_or(fail);
+    if (!failed && rank == 0 && lane == 0) *a.t = t;
+    cluster_sync();  // no block pushes any more, and s_sent is complete
+    if (failed) {
+      bool drained = true;
+#pragma unroll
+      for (unsigned b = 0; b < 2; ++b) {
+        const unsigned e = armed_ring - b, m = armed_min - b;
+        unsigned missing = 0u;  // bytes of epoch e that were never sent
+        for (int r = lane; r < info.y; r += 32) {
+          const int i = __ldg(a.ring_id + info.x + r);
+          if (s_sent[index_ok(i, a.n, a.err) ? i / a.tile : rank].x < e) missing += 16u;
+        }
+        missing = __reduce_add_sync(0xffffffffu, missing);
+        if (lane == 0 && missing) forgo_tx(&ring_bar[e & 1u], missing);
+        const unsigned silent = __popc(
+            __ballot_sync(0xffffffffu, lane < blocks && s_sent[lane % kLoopMaxTiles].y <= m));
+        if (lane == 0 && silent) forgo_tx(&min_bar[m & 1u], silent * kWarps * 4u);
+        __syncwarp();
+        drained = await(&ring_bar[e & 1u], ((e - 1u) >> 1) & 1u, a.drain_polls) && drained;
+        drained = await(&min_bar[m & 1u], (m >> 1) & 1u, a.drain_polls) && drained;
+      }
+      if (!drained) atomicOr(a.err, 4);
+    }
     return;
   }
 
@@ -203,6 +249,7 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
   const int edges = info.z;
   float4* const base = s0;
   unsigned epoch = 0u;  // of the states now read
+  unsigned pushed = 0u;  // the last epoch this block's edge cells were pushed of
 
   LoopCell c{};
   const bool has = tid < nt;
@@ -320,14 +367,17 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
     constexpr int kFirst = RK2 ? kModeRK2a : kModeFE;
     if (has) finish(std::integral_constant<int, kFirst>{}, s0, s1, dt, RK2 || !last);
     ++epoch;
+    if (RK2 || !last) pushed = epoch;
     if (RK2) {
-      __syncthreads();  // B: U* of the tile is complete
       await_ring();
+      stop = __syncthreads_or(fail);  // B: U* of the tile and its ring is complete
+      if (stop) break;
       if (has) {
         fluxes(s1);
         finish(std::integral_constant<int, kModeRK2b>{}, s1, s0, dt, !last);
       }
       ++epoch;
+      if (!last) pushed = epoch;
     } else {
       float4* s = s0;
       s0 = s1;
@@ -348,6 +398,7 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
     }
     if (!ok) atomicOr(a.err, 1);
   }
+  if (warp == 0 && lane < blocks) store_remote(remote(&s_sent[rank], lane), pushed, minima);
   cluster_sync();  // no block leaves while another may still write to it
 }
 
