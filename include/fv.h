@@ -83,6 +83,15 @@ extern "C" {
 #define FV_WAVE_AVERAGE 0 /* |average normal velocity| + average sound speed (Sec. 6.2.2) */
 #define FV_WAVE_MAX 1     /* max over both sides of |normal velocity| + sound speed */
 
+/* What fv_mesh_get_step_kernel and fv_batch_get_step_kernel report beside the
+ * shapes 0-7 of fv_mesh_set_variant */
+#define FV_KERNEL_NONE (-1)
+#define FV_KERNEL_LOOP 8
+#define FV_KERNEL_ONE_WAVE 9
+#define FV_KERNEL_PAIRS 10
+#define FV_KERNEL_LEARNED 11
+#define FV_KERNEL_LEARNED_TILES 12
+
 typedef struct fv_mesh fv_mesh;
 typedef struct fv_batch fv_batch;
 typedef struct fv_closure fv_closure;
@@ -213,6 +222,10 @@ int fv_mesh_set_variant(fv_mesh* mesh, int32_t variant);
  * fastest for later fv_step calls and reports it in *best (nullable);
  * us_per_step (nullable, host, [8]) receives the measured microseconds per
  * step of each shape (infinity for a tiled shape when its tiles do not fit).
+ * On a mesh that the resident loop takes (see fv_step) the loop is timed too and,
+ * where it is faster than every shape, run by later fv_step calls; *best and
+ * us_per_step are the shapes' all the same (fv_mesh_get_step_kernel tells which
+ * ran).
  * Shapes 6 and 7 are timed with tiles of 256, 384, 512, 768, 1024 and 2048
  * cells (and sizes that fill whole waves) and reported at their best; when one wins, its
  * tile size is kept (the tile size is shared with fv_mesh_set_blocking).  Allocates and frees one state-sized device buffer
@@ -331,10 +344,25 @@ int fv_mesh_set_launch_chaining(fv_mesh* mesh, int32_t enable);
 int fv_mesh_set_blocking(fv_mesh* mesh, int32_t steps_per_launch, int32_t tile_cells,
                          int32_t staged);
 
-/* The step-kernel shape (0-6) and the tile size in cells of the tiled shapes
- * that the mesh runs now (set by fv_mesh_set_variant, fv_mesh_set_blocking,
- * fv_mesh_set_geometry or fv_mesh_autotune).  Outputs nullable, host. */
+/* The step-kernel shape (0-7) and the tile size in cells of the tiled shapes
+ * that are set for the mesh (by fv_mesh_set_variant, fv_mesh_set_blocking,
+ * fv_mesh_set_geometry or fv_mesh_autotune; 1 and 1024 before).  Where none was
+ * set, and where the autotuner found the resident loop faster than every shape,
+ * fv_step runs something else: fv_mesh_get_step_kernel tells.  Outputs nullable,
+ * host. */
 int fv_mesh_get_tiling(const fv_mesh* mesh, int32_t* variant, int32_t* tile_cells);
+
+/* What the mesh's last fv_step (of at least one step and one cell) ran.
+ *   kernel      a shape 0-7 (fv_mesh_set_variant), FV_KERNEL_LOOP (the whole
+ *               time loop in one launch of one cluster), FV_KERNEL_ONE_WAVE (the
+ *               form of shape 6 whose tiles are all resident at a time),
+ *               FV_KERNEL_PAIRS (two steps per launch), FV_KERNEL_LEARNED (a
+ *               pass for the closure's scales and a step that reads them),
+ *               FV_KERNEL_LEARNED_TILES (the learned step in one kernel), or
+ *               FV_KERNEL_NONE before the first step.
+ *   tile_cells  cells of its tiles, 0 for a kernel without tiles.
+ * Outputs nullable, host. */
+int fv_mesh_get_step_kernel(const fv_mesh* mesh, int32_t* kernel, int32_t* tile_cells);
 
 /* Host diagnostics of the two-step tiles: the halos of tile `tile` (cells
  * [tile*tile_cells, (tile+1)*tile_cells) of the current numbering).
@@ -549,8 +577,13 @@ int fv_batch_info(const fv_batch* batch, int64_t* n_cells_padded, int64_t* offse
 int fv_batch_set_variant(fv_batch* batch, int32_t variant);
 
 /* The batch's kernel shape in *variant: 0, 5 or 6, or -1 while the default
- * is still to be decided at the first device call. */
+ * is still to be decided at the first device call.  The shape that the steps
+ * run while none is set: fv_batch_get_step_kernel. */
 int fv_batch_get_variant(const fv_batch* batch, int32_t* variant);
+
+/* The shape the batch's last fv_batch_step (of at least one step) ran: 0, 5 or
+ * 6, or FV_KERNEL_NONE before the first. */
+int fv_batch_get_step_kernel(const fv_batch* batch, int32_t* kernel);
 
 /* Compensated float update for FV_F32 batches (see fv_mesh_set_compensation). */
 int fv_batch_set_compensation(fv_batch* batch, int32_t enable);

@@ -21,6 +21,8 @@ FV_F32, FV_F64 = 0, 1
 FV_BC_NONE, FV_BC_WALL, FV_BC_FARFIELD, FV_BC_EXTRAP = 0, 1, 2, 3
 ORDERS = {"identity": 0, "shuffle": 1, "rcm": 2, "hilbert": 3, "am1": 4}
 SCHEMES = {"fe": 0, "rk2": 1}
+# what step_kernel() reports beside the shapes
+(KERNEL_LOOP, KERNEL_ONE_WAVE, KERNEL_PAIRS, KERNEL_LEARNED, KERNEL_LEARNED_TILES) = range(8, 13)
 
 _lock = threading.Lock()
 _lib = None
@@ -80,6 +82,7 @@ def load():
             "fv_mesh_set_closure_engine": (ctypes.c_int, [_vp, _i32]),
             "fv_mesh_set_geometry": (ctypes.c_int, [_vp, _i32]),
             "fv_mesh_get_tiling": (ctypes.c_int, [_vp, _P(_i32), _P(_i32)]),
+            "fv_mesh_get_step_kernel": (ctypes.c_int, [_vp, _P(_i32), _P(_i32)]),
             "fv_mesh_tile_nodes": (ctypes.c_int, [_vp, _i32, _i64, _vp, _i64, _P(_i64), _vp]),
             "fv_mesh_nodes": (ctypes.c_int, [_vp, _P(_i64), _vp, _P(_i32)]),
             "fv_mesh_tile_halo": (ctypes.c_int, [_vp, _i32, _i64, _vp, _i64, _P(_i64), _P(_i64)]),
@@ -108,6 +111,7 @@ def load():
             "fv_batch_set_remainder": (ctypes.c_int, [_vp, _vp]),
             "fv_batch_set_variant": (ctypes.c_int, [_vp, _i32]),
             "fv_batch_get_variant": (ctypes.c_int, [_vp, _P(_i32)]),
+            "fv_batch_get_step_kernel": (ctypes.c_int, [_vp, _P(_i32)]),
             "fv_batch_step": (ctypes.c_int, [_vp, _vp, _i64, _dbl, _dbl, _i32, _vp, _vp]),
             "fv_batch_totals": (ctypes.c_int, [_vp, _vp, _vp, _vp]),
         }
@@ -317,9 +321,16 @@ class Mesh:
         return q[:nn.value].copy(), loc[:cells].copy()
 
     def tiling(self):
-        """(step-kernel shape, tile size in cells of the tiled shapes)."""
+        """(step-kernel shape, tile size in cells of the tiled shapes), as set."""
         v, t = _i32(), _i32()
         _check(load().fv_mesh_get_tiling(self._h, ctypes.byref(v), ctypes.byref(t)))
+        return int(v.value), int(t.value)
+
+    def step_kernel(self):
+        """(kernel, tile size in cells) of the last step call: a shape 0-7 or
+        KERNEL_*; (-1, 0) before the first."""
+        v, t = _i32(), _i32()
+        _check(load().fv_mesh_get_step_kernel(self._h, ctypes.byref(v), ctypes.byref(t)))
         return int(v.value), int(t.value)
 
     def tile_halo(self, tile_cells: int, tile: int):
@@ -512,6 +523,12 @@ class Batch:
         """Kernel shape of the batch (-1 until the first device call)."""
         v = _i32()
         _check(load().fv_batch_get_variant(self._h, ctypes.byref(v)))
+        return int(v.value)
+
+    def step_kernel(self) -> int:
+        """Shape of the last step call (-1 before the first)."""
+        v = _i32()
+        _check(load().fv_batch_get_step_kernel(self._h, ctypes.byref(v)))
         return int(v.value)
 
     def step(self, U, nsteps, cfl, t_stop=0.0, scheme="fe", stream=None, sync=True):

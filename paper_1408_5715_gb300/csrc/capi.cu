@@ -209,6 +209,7 @@ struct fv_mesh {
   bool g_chained = false;
   int last_t_slot = 0;
   bool stepped = false;
+  int ran_kernel = FV_KERNEL_NONE, ran_tile = 0;  // fv_mesh_get_step_kernel
 
   bool f64() const { return precision == FV_F64; }
   size_t rec_bytes() const { return f64() ? 32 : 16; }
@@ -903,6 +904,24 @@ void capture_graph(fv_mesh* m, void* U, double cfl, double t_stop, int32_t schem
   m->g_chained = m->chained;
 }
 
+// Notes what a launch per step (or pair of steps) runs (fv_mesh_get_step_kernel).
+void note_kernel(fv_mesh* m, const fv_closure* cl) {
+  int k = m->shape();
+  if (m->blocking == 2) {
+    k = FV_KERNEL_PAIRS;
+  } else if (cl) {
+    k = m->variant == fv::kFaceTileVariant ? FV_KERNEL_LEARNED_TILES : FV_KERNEL_LEARNED;
+  } else if (k == fv::kTileVariant && m->tiles_quick && !m->tiles_vertex) {
+    k = FV_KERNEL_ONE_WAVE;
+  } else if (m->wave == FV_WAVE_MAX && k >= 2 && k <= 5) {
+    k = 1;
+  }
+  const bool tiled = tiled_shape(k) || k == FV_KERNEL_ONE_WAVE || k == FV_KERNEL_PAIRS ||
+                     k == FV_KERNEL_LEARNED_TILES;
+  m->ran_kernel = k;
+  m->ran_tile = tiled ? m->tiles_built : 0;
+}
+
 void read_status(fv_mesh* m, cudaStream_t s, double* t_adv, bool check) {
   fv::LoopScalars h{};
   FV_CUDA(cudaMemcpyAsync(&h, m->d_scal, sizeof h, cudaMemcpyDeviceToHost, s));
@@ -1099,6 +1118,14 @@ int fv_mesh_get_tiling(const fv_mesh* mesh, int32_t* variant, int32_t* tile_cell
     check_mesh(mesh);
     if (variant) *variant = mesh->variant;
     if (tile_cells) *tile_cells = mesh->pair_tile;
+  });
+}
+
+int fv_mesh_get_step_kernel(const fv_mesh* mesh, int32_t* kernel, int32_t* tile_cells) {
+  return guarded([&] {
+    check_mesh(mesh);
+    if (kernel) *kernel = mesh->ran_kernel;
+    if (tile_cells) *tile_cells = mesh->ran_tile;
   });
 }
 
@@ -1420,6 +1447,8 @@ int fv_step(fv_mesh* mesh, void* U, int64_t nsteps, double cfl, double t_stop, i
     mesh->stepped = true;
     if (n > 0 && nsteps > 0 && uses_loop(mesh, closure)) {
       if (mesh->blocking == 2) check_tile_smem(mesh, pair_smem(mesh));
+      mesh->ran_kernel = FV_KERNEL_LOOP;
+      mesh->ran_tile = mesh->loop_tile;
       const bool keep = mesh->use_lo() && mesh->user_lo;
       if (keep)  // the remainder the caller kept from the last call
         FV_CUDA(cudaMemcpyAsync(mesh->d_lo, mesh->user_lo, n * sizeof(uint2),
@@ -1433,6 +1462,7 @@ int fv_step(fv_mesh* mesh, void* U, int64_t nsteps, double cfl, double t_stop, i
     }
     FV_CUDA(fv::launch_init_scalars(mesh->d_scal, s));
     if (n > 0 && nsteps > 0) {
+      note_kernel(mesh, closure);
       if (mesh->use_lo()) {
         if (mesh->user_lo)  // the remainder the caller kept from the last call
           FV_CUDA(cudaMemcpyAsync(mesh->d_lo, mesh->user_lo, n * sizeof(uint2),
@@ -1587,6 +1617,7 @@ struct fv_batch {
   bool shape_chosen = false;
   int auto_variant = 0;
   int shape() const { return shape_chosen ? variant : auto_variant; }
+  int ran_kernel = FV_KERNEL_NONE;  // fv_batch_get_step_kernel
   // shared-memory tiles of 1024 cells within each mesh (shape 6)
   bool tiles_ok = false;
   int32_t t1_cap = 0;
@@ -2001,6 +2032,14 @@ int fv_batch_set_remainder(fv_batch* batch, void* lo) {
   });
 }
 
+int fv_batch_get_step_kernel(const fv_batch* batch, int32_t* kernel) {
+  return guarded([&] {
+    check_batch(batch);
+    if (!kernel) invalid("null kernel");
+    *kernel = batch->ran_kernel;
+  });
+}
+
 int fv_batch_step(fv_batch* batch, void* U, int64_t nsteps, double cfl, double t_stop,
                   int32_t scheme, void* stream, double* t_advanced) {
   return guarded([&] {
@@ -2017,6 +2056,7 @@ int fv_batch_step(fv_batch* batch, void* U, int64_t nsteps, double cfl, double t
     batch->last_t_slot = 0;
     batch->stepped = true;
     if (nsteps > 0) {
+      batch->ran_kernel = batch->shape();
       if (batch->use_lo()) {
         if (batch->user_lo)
           FV_CUDA(cudaMemcpyAsync(batch->d_lo, batch->user_lo, batch->n * sizeof(uint2),
