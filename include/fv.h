@@ -439,7 +439,10 @@ int fv_mesh_debug_set_index(fv_mesh* mesh, int32_t table, int64_t cell, int32_t 
  * FV_F32 meshes of up to 12,288 cells whose kernel shape was not chosen
  * (fv_mesh_set_variant) and that step without a closure run the whole loop in
  * one launch on one thread-block cluster instead (also with two steps per
- * launch, when their tile size was left to the library); same bits. */
+ * launch, when their tile size was left to the library); same bits.
+ * In a stream that the caller captures, a mesh without a chosen shape steps on
+ * shape 0 or 1, whose arrays only fv_renumber and fv_mesh_destroy change: the
+ * captured steps stay valid whatever shape is set later. */
 int fv_step(fv_mesh* mesh, void* U, int64_t nsteps, double cfl, double t_stop, int32_t scheme,
             const fv_closure* closure, void* stream, double* t_advanced);
 

@@ -139,7 +139,15 @@ struct fv_mesh {
   // one by the mesh's size (choose_shape, when the device arrays are made).
   bool shape_chosen = false;
   int auto_variant = 1, auto_tile = 0;
-  int shape() const { return shape_chosen || blocking == 2 ? variant : auto_variant; }
+  // True inside an fv_step that the caller captures: a graph of its own may be
+  // replayed after the library's tables changed with a later choice or order, so
+  // the default paths do without tables then.
+  bool captured = false;
+  // the default shape without tables (choose_shape)
+  int plain_shape() const { return !f64() && h.n <= 230000 ? 0 : 1; }
+  int shape() const {
+    return shape_chosen || blocking == 2 ? variant : captured ? plain_shape() : auto_variant;
+  }
   int shape_tile() const {
     return shape_chosen || blocking == 2 || auto_tile == 0 ? pair_tile : auto_tile;
   }
@@ -560,11 +568,10 @@ void choose_shape(fv_mesh* m, cudaStream_t s) {
     good = good && (m->f64() ? 2 * m->tiles_halo_cells <= 5 * n
                              : m->tiles_quick && 4 * m->tiles_halo_cells <= 3 * n);
     if (good) return;
-    m->auto_variant = 1;
     m->auto_tile = 0;
     m->free_tiles();
   }
-  if (!m->f64() && n <= 230000) m->auto_variant = 0;
+  m->auto_variant = m->plain_shape();
 }
 
 void ensure_device(fv_mesh* m, cudaStream_t s) {
@@ -831,7 +838,7 @@ void enqueue_launches(fv_mesh* m, void* U, int64_t j0, int64_t launches, double 
 // asks for a kernel shape of its own, and with two steps per launch the tile
 // size was left to the library.
 bool uses_loop(const fv_mesh* m, const fv_closure* cl) {
-  if (m->loop_tiles == 0 || cl || m->vertex_tiles()) return false;
+  if (m->loop_tiles == 0 || cl || m->vertex_tiles() || m->captured) return false;
   return m->blocking == 2 ? m->pair_default : m->loop_wanted;
 }
 
@@ -1440,6 +1447,11 @@ int fv_step(fv_mesh* mesh, void* U, int64_t nsteps, double cfl, double t_stop, i
       invalid("the maximum wave speed runs without a closure, one step per launch");
     if (!U && nsteps > 0 && mesh->h.n > 0) invalid("null state");
     cudaStream_t s = as_stream(stream);
+    mesh->captured = capturing(s);
+    struct Reset {
+      fv_mesh* m;
+      ~Reset() { m->captured = false; }
+    } reset{mesh};
     ensure_device(mesh, s);
     if (closure) ensure_faces(mesh, s);
     const int64_t n = mesh->h.n;
