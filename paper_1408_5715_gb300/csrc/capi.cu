@@ -136,8 +136,9 @@ struct fv_mesh {
   void* user_lo = nullptr;      // caller-owned remainder (fv_mesh_set_remainder)
   int variant = 1;              // step-kernel shape (fv_mesh_autotune / fv_mesh_set_variant)
   // While no shape was chosen (and one step runs per launch) the library takes
-  // one by the mesh's size (choose_shape, when the device arrays are made).
+  // one by the mesh's size (choose_shape, at the first step that asks for it).
   bool shape_chosen = false;
+  bool auto_known = false;
   int auto_variant = 1, auto_tile = 0;
   // True inside an fv_step that the caller captures: a graph of its own may be
   // replayed after the library's tables changed with a later choice or order, so
@@ -186,11 +187,11 @@ struct fv_mesh {
   fv::FaceRec* d_faces = nullptr;
   int64_t n_faces = 0;
   float* d_scale = nullptr;
-  // the resident loop (loop_step.cu): tiles of the whole-loop kernel, built
-  // with the device arrays when one cluster holds the mesh (loop_tiles = 0: not).
-  // It runs where no shape was chosen, or the autotuner found it faster than
-  // every shape (loop_wanted).
-  bool loop_wanted = true;
+  // the resident loop (loop_step.cu): tiles of the whole-loop kernel, built by
+  // the first call that may run it (loop_known) when one cluster holds the mesh
+  // (loop_tiles = 0: not).  It runs where no shape was chosen, or the autotuner
+  // found it faster than every shape (loop_wanted).
+  bool loop_wanted = true, loop_known = false;
   int loop_tile = 0, loop_tiles = 0, loop_cap = 0;
   unsigned char* d_loop = nullptr;  // holds the arrays below
   float4* loop_geom = nullptr;
@@ -252,6 +253,11 @@ struct fv_mesh {
   }
 
   bool vertex_tiles() const { return geometry == FV_GEOM_VERTEX; }
+  // a shape or two steps per launch was set that runs on tiles
+  bool set_tiles() const {
+    return blocking == 2 ||
+           (shape_chosen && (variant == fv::kTileVariant || variant == fv::kFaceTileVariant));
+  }
 
   void free_faces() {
     dev_free(d_faces);
@@ -264,11 +270,19 @@ struct fv_mesh {
     loop_tile = loop_tiles = loop_cap = 0;
   }
 
+  // back to no choice of the library's (new device arrays or a new order)
+  void drop_defaults() {
+    free_loop();
+    loop_known = auto_known = false;
+    auto_variant = 1;
+    auto_tile = 0;
+  }
+
   void free_device() {
     drop_graph();
     free_tiles();
     free_faces();
-    free_loop();
+    drop_defaults();
     dev_free(d_nbr);
     dev_free(d_geom);
     dev_free(d_vol);
@@ -553,10 +567,7 @@ void build_loop(fv_mesh* m, cudaStream_t s) {
 //   the cells, then shape 0 (160,000: 3.5 against 3.9 for shape 1) up to
 //   230,000 (250,000: 5.3 against 4.8), then shape 1.
 void choose_shape(fv_mesh* m, cudaStream_t s) {
-  m->auto_variant = 1;
-  m->auto_tile = 0;
   const int64_t n = m->h.n;
-  if (m->shape_chosen || m->blocking == 2 || m->loop_tiles > 0 || n == 0) return;
   const bool tiled = m->f64() || n <= 90000;
   if (tiled) {
     m->auto_variant = m->f64() ? fv::kFaceTileVariant : fv::kTileVariant;
@@ -581,11 +592,12 @@ void ensure_device(fv_mesh* m, cudaStream_t s) {
     invalid("mesh was uploaded to device " + std::to_string(m->device) +
             " but the current device is " + std::to_string(dev));
   if (!m->dirty && m->dev_n == m->h.n) {
-    ensure_tiles(m, s);
+    if (m->set_tiles()) ensure_tiles(m, s);
     return;
   }
   m->free_tiles();
   m->free_faces();
+  m->drop_defaults();
   const int64_t n = m->h.n;
   if (m->dev_n != n) {
     m->free_device();
@@ -616,13 +628,46 @@ void ensure_device(fv_mesh* m, cudaStream_t s) {
     FV_CUDA(cudaMemcpyAsync(m->d_vol, m->h.vol.data(), n * sizeof(double), cudaMemcpyHostToDevice,
                             s));
     FV_CUDA(cudaStreamSynchronize(s));  // lay is a local staging buffer
-    if (!optional_tables([&] { build_loop(m, s); })) m->free_loop();
   }
   FV_CUDA(cudaStreamSynchronize(s));
   m->device = dev;
   m->dirty = false;
-  choose_shape(m, s);
-  ensure_tiles(m, s);
+  if (m->set_tiles()) ensure_tiles(m, s);
+}
+
+// Whether one cluster holds the mesh: builds the loop's tables once.
+void ensure_loop(fv_mesh* m, cudaStream_t s) {
+  if (m->loop_known) return;
+  m->loop_known = true;
+  if (!optional_tables([&] { build_loop(m, s); })) m->free_loop();
+}
+
+// Whether nothing asks for a kernel shape of its own where the resident loop
+// may run (with two steps per launch: the tile size was left to the library).
+bool wants_loop(const fv_mesh* m, const fv_closure* cl) {
+  if (cl || m->vertex_tiles() || m->captured) return false;
+  return m->blocking == 2 ? m->pair_default : m->loop_wanted;
+}
+
+bool uses_loop(const fv_mesh* m, const fv_closure* cl) {
+  return m->loop_tiles > 0 && wants_loop(m, cl);
+}
+
+// What the default paths need, at the first step that takes them: a mesh that
+// is only monitored or trained on, or whose shape is set, neither builds nor
+// holds it.
+void ensure_default(fv_mesh* m, cudaStream_t s) {
+  if (m->captured) return;
+  if (wants_loop(m, nullptr)) ensure_loop(m, s);
+  if (m->shape_chosen || m->blocking == 2 || uses_loop(m, nullptr)) return;
+  if (!m->auto_known) choose_shape(m, s);
+  m->auto_known = true;
+  // tiles of another size may have taken the place of the default shape's
+  if (!optional_tables([&] { ensure_tiles(m, s); })) {
+    m->free_tiles();
+    m->auto_variant = m->plain_shape();
+    m->auto_tile = 0;
+  }
 }
 
 // The faces of the mesh, each once, for the learned closure's scale pass:
@@ -832,14 +877,6 @@ void enqueue_launches(fv_mesh* m, void* U, int64_t j0, int64_t launches, double 
     enqueue_pairs(m, U, j0, launches, cfl, t_stop, s);
   else
     enqueue_steps(m, U, j0, launches, cfl, t_stop, scheme, s, cl);
-}
-
-// Whether fv_step runs the resident loop: the mesh has its tiles, nothing
-// asks for a kernel shape of its own, and with two steps per launch the tile
-// size was left to the library.
-bool uses_loop(const fv_mesh* m, const fv_closure* cl) {
-  if (m->loop_tiles == 0 || cl || m->vertex_tiles() || m->captured) return false;
-  return m->blocking == 2 ? m->pair_default : m->loop_wanted;
 }
 
 // Enqueues nsteps of the resident loop.  The remainders start from lo_in
@@ -1319,6 +1356,7 @@ int fv_mesh_autotune(fv_mesh* mesh, const void* U, int32_t scheme, void* stream,
       // the resident loop against them, over the same steps
       mesh->blocking = 1;
       mesh->loop_wanted = true;
+      if (wants_loop(mesh, nullptr)) ensure_loop(mesh, s);
       if (uses_loop(mesh, nullptr)) {
         FV_CUDA(cudaMemcpyAsync(tmp, U, n * mesh->rec_bytes(), cudaMemcpyDeviceToDevice, s));
         enqueue_loop(mesh, tmp, 2, cfl, 0.0, scheme, nullptr, s);
@@ -1455,6 +1493,7 @@ int fv_step(fv_mesh* mesh, void* U, int64_t nsteps, double cfl, double t_stop, i
     ensure_device(mesh, s);
     if (closure) ensure_faces(mesh, s);
     const int64_t n = mesh->h.n;
+    if (!closure && n > 0 && nsteps > 0) ensure_default(mesh, s);
     mesh->last_t_slot = 0;
     mesh->stepped = true;
     if (n > 0 && nsteps > 0 && uses_loop(mesh, closure)) {
