@@ -172,7 +172,6 @@ struct fv_mesh {
   int p_f_cap = 0;
   int p_e_cap = 0, p_t1_cap = 0;
   bool tiles_pairs = false;        // the tiles have their second halos
-  int64_t tiles_halo_cells = 0;    // halo entries of all tiles
   bool tiles_quick = false;  // FP32: the one-step tiles are all resident at a time
   // normals from vertex coordinates (fv_mesh_set_geometry): tile nodes
   int geometry = FV_GEOM_STORED;
@@ -364,23 +363,11 @@ void upload_tile_faces(fv_mesh* m, const fv::PairTiles& L, cudaStream_t s) {
   FV_CUDA(cudaStreamSynchronize(s));  // L and st are staging buffers
 }
 
-void ensure_tiles(fv_mesh* m, cudaStream_t s) {
-  if (!uses_tiles(m) || m->h.n == 0) return;
-  const int tile = m->shape_tile();
+// The tiles L of the mesh's shape and tile size on the device
+// (free_tiles and drop_graph before it); faces: for shape 7.
+void upload_tiles(fv_mesh* m, fv::PairTiles& L, bool faces, cudaStream_t s) {
+  const int tile = L.tile;
   const bool pairs = m->blocking == 2;
-  const bool faces = m->shape() == fv::kFaceTileVariant && !m->vertex_tiles();
-  if (m->tiles_built == tile && m->tiles_vertex == m->vertex_tiles() &&
-      (m->tiles_pairs || !pairs)) {
-    if (faces && !m->d_face_rec) {
-      m->drop_graph();
-      upload_tile_faces(m, fv::build_step_tiles(m->h, tile, true), s);
-    }
-    return;
-  }
-  m->free_tiles();
-  m->drop_graph();
-  fv::PairTiles L =
-      pairs ? fv::build_pair_tiles(m->h, tile) : fv::build_step_tiles(m->h, tile, faces);
   if (faces) upload_tile_faces(m, L, s);
   fv::TileVertices V;
   if (m->vertex_tiles()) {
@@ -421,8 +408,27 @@ void ensure_tiles(fv_mesh* m, cudaStream_t s) {
   m->p_v_cap = V.v_cap;
   m->tiles_vertex = m->vertex_tiles();
   m->tiles_pairs = pairs;
-  m->tiles_halo_cells = (int64_t)L.halo_id.size();
   m->tiles_built = tile;
+}
+
+void ensure_tiles(fv_mesh* m, cudaStream_t s) {
+  if (!uses_tiles(m) || m->h.n == 0) return;
+  const int tile = m->shape_tile();
+  const bool pairs = m->blocking == 2;
+  const bool faces = m->shape() == fv::kFaceTileVariant && !m->vertex_tiles();
+  if (m->tiles_built == tile && m->tiles_vertex == m->vertex_tiles() &&
+      (m->tiles_pairs || !pairs)) {
+    if (faces && !m->d_face_rec) {
+      m->drop_graph();
+      upload_tile_faces(m, fv::build_step_tiles(m->h, tile, true), s);
+    }
+    return;
+  }
+  m->free_tiles();
+  m->drop_graph();
+  fv::PairTiles L =
+      pairs ? fv::build_pair_tiles(m->h, tile) : fv::build_step_tiles(m->h, tile, faces);
+  upload_tiles(m, L, faces, s);
 }
 
 // Shared memory of the one-step tile kernel of this mesh.
@@ -557,32 +563,57 @@ void build_loop(fv_mesh* m, cudaStream_t s) {
   m->loop_cap = L.cap;
 }
 
+// Device bytes of an FP64 mesh's shape-7 tables: 32 for each of 3/2 faces a
+// cell, 8 for the faces' words, 16 a cell for neighbours and references, and
+// the rings.
+size_t fp64_table_bytes(int64_t n) { return (size_t)n * 80; }
+
+// Whether tables of so many bytes take a small share of what the device has
+// left.  The caller's arrays come first: tables beyond 64 MB are made only
+// where eight times as much is free.
+bool leaves_memory(size_t bytes) {
+  if (bytes <= (size_t)64 << 20) return true;
+  size_t free = 0, total = 0;
+  FV_CUDA(cudaMemGetInfo(&free, &total));
+  return free / 8 >= bytes;
+}
+
 // The step-kernel shape of a mesh whose shape was not chosen, by size
 // (measured us per step, forward Euler):
 //   FP64: shape 7 (102,400 cells: 24.5 against 52 for shape 1; 12,800: 9.4
 //   against 19.2), whose tiles must be compact: with rings of more than 2.5
 //   times the tile a face evaluated once no longer pays for staging the ring;
+//   else shape 1, which needs no tables;
 //   FP32: up to 90,000 cells the one-wave tiles (65,536: 2.4 against 2.6 for
 //   shape 0, 102,400: 3.1 against 2.8) when their rings hold less than 3/4 of
 //   the cells, then shape 0 (160,000: 3.5 against 3.9 for shape 1) up to
 //   230,000 (250,000: 5.3 against 4.8), then shape 1.
 void choose_shape(fv_mesh* m, cudaStream_t s) {
   const int64_t n = m->h.n;
-  const bool tiled = m->f64() || n <= 90000;
-  if (tiled) {
-    m->auto_variant = m->f64() ? fv::kFaceTileVariant : fv::kTileVariant;
-    m->auto_tile = (int)(m->f64() ? fp64_tile(n) : quick_tile(n));
-    bool good = optional_tables([&] {
-      ensure_tiles(m, s);
-      check_tile_smem(m, step_tile_smem(m));
-    });
-    good = good && (m->f64() ? 2 * m->tiles_halo_cells <= 5 * n
-                             : m->tiles_quick && 4 * m->tiles_halo_cells <= 3 * n);
-    if (good) return;
-    m->auto_tile = 0;
-    m->free_tiles();
-  }
   m->auto_variant = m->plain_shape();
+  m->auto_tile = 0;
+  if (!m->f64() && n > 90000) return;
+  const int tile = (int)(m->f64() ? fp64_tile(n) : quick_tile(n));
+  bool good = m->f64() ? leaves_memory(fp64_table_bytes(n)) : true;
+  good = good && optional_tables([&] {
+    fv::PairTiles L = fv::build_step_tiles(m->h, tile, m->f64());
+    const int64_t rings = (int64_t)L.halo_id.size();
+    if (m->f64() ? 2 * rings > 5 * n
+                 : 4 * rings > 3 * n || !fv::tile_quick_fits(n, tile, L.t1_cap))
+      invalid("tiles not worth their rings");
+    check_tile_smem(m, m->f64() ? fv::tile_faces_smem_bytes(true, L.t1_cap, tile, L.f_cap)
+                                : fv::tile_smem_bytes(false, L.t1_cap));
+    m->free_tiles();
+    m->drop_graph();
+    upload_tiles(m, L, m->f64(), s);
+  });
+  if (good) {
+    m->auto_variant = m->f64() ? fv::kFaceTileVariant : fv::kTileVariant;
+    m->auto_tile = tile;
+  } else {
+    m->free_tiles();
+    m->drop_graph();
+  }
 }
 
 void ensure_device(fv_mesh* m, cudaStream_t s) {
