@@ -23,11 +23,12 @@
 // last one.
 //
 // Waits are bounded.  A block in which one gives up (error bit 2) stops as a
-// whole at the barrier that follows every wait, so it has pushed its stages
-// whole or not at all, and the blocks that wait for it give up in turn.  Every
-// block leaves the number of stages it pushed with all others before the
-// closing cluster barrier; one that gave up then knows which stores are still
-// on their way to it and awaits those (drain) before it leaves.
+// whole at the next barrier of dt, so it has pushed its stages whole or not at
+// all, and the blocks that wait for it give up in turn.  Every block leaves the
+// number of stages it pushed with all others before the closing cluster
+// barrier; one that gave up then knows which stores are still on their way to
+// it and awaits those (drain) before it leaves.  (Stopping at a vote behind the
+// wait for RK2's first stage too cost 3-7 % of a step.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -73,7 +74,8 @@ __device__ __forceinline__ void push_value(unsigned to, float v, unsigned bar) {
 __device__ __forceinline__ void store_remote(unsigned to, unsigned x, unsigned y) {
   asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(to), "r"(x), "r"(y) : "memory");
 }
-// Takes bytes that will not come off what an mbarrier of this block expects.
+// Takes bytes that will not come off what an mbarrier of this block expects
+// (in the pieces they would have come in, so that no sum jumps over zero).
 __device__ __forceinline__ void forgo_tx(uint64_t* bar, unsigned bytes) {
   asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)),
                "r"(bytes)
@@ -159,8 +161,8 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
   cluster_sync();  // every block's mbarriers are ready
 
   if (warp == kWarps) {
-    // ring epochs 1, 2, ... (states after each stage), minima 0, 1, ...; of
-    // each kind the last two armed may be under way
+    // ring epochs 1, 2, ... (states after each stage), minima 0, 1, ...: the
+    // last one armed of each (and with it the one before)
     unsigned armed_ring = 2u, armed_min = 1u;
     if (lane == 0) {
       mbar_expect_tx(&ring_bar[1], ring_bytes);
@@ -170,22 +172,23 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
     }
     double dt_raw = 0.0;
     unsigned epoch = 0u, minima = 0u;
-    // every compute thread has awaited this epoch's ring (they passed the
-    // barrier after that wait): its mbarrier is armed for the one after next
-    auto rearm_ring = [&]() {
-      if (lane == 0) mbar_expect_tx(&ring_bar[epoch & 1u], ring_bytes);
-      armed_ring = epoch + 2u;
+    // Behind the barrier of dt every thread has been through the waits before
+    // it: their mbarriers are armed for the epoch after next (what a quick block
+    // has already sent of that one only counts the bytes below zero meanwhile).
+    auto rearm = [&](bool due) {
+      if (lane == 0) {
+        if (due) mbar_expect_tx(&min_bar[(minima + 1u) & 1u], min_bytes);
+        if (epoch > 0u && RK2) mbar_expect_tx(&ring_bar[1], ring_bytes);
+        if (epoch > 0u) mbar_expect_tx(&ring_bar[RK2 ? 0u : epoch & 1u], ring_bytes);
+      }
+      if (due) armed_min = minima + 1u;
+      if (epoch > 0u) armed_ring = epoch + 2u;
     };
     bool due = true;
     for (int j = 0; j < a.nsteps; ++j) {
       if (due) {
         const unsigned p = minima & 1u;
-        if (__all_sync(0xffffffffu, await(&min_bar[p], (minima >> 1) & 1u, a.polls))) {
-          armed_min = minima + 2u;
-          if (lane == 0) mbar_expect_tx(&min_bar[p], min_bytes);
-        } else {
-          fail = true;
-        }
+        if (!await(&min_bar[p], (minima >> 1) & 1u, a.polls)) fail = true;
         float m = INFINITY;
 #pragma unroll
         for (int k = 0; k < kRow / 128; ++k) {
@@ -206,14 +209,10 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
       if (lane == 0) s_dt = (float)dt;
       if (__syncthreads_or(fail)) break;  // C: dt is there, the ring was awaited
       t += dt;
+      rearm(due);
       due = a.steps_per_bound == 1 || !due;
-      if (epoch > 0u) rearm_ring();  // the ring this step reads
-      ++epoch;
-      if (RK2) {
-        if (__syncthreads_or(fail)) break;  // B: U*'s ring was awaited
-        rearm_ring();
-        ++epoch;
-      }
+      epoch += RK2 ? 2u : 1u;
+      if (RK2) __syncthreads();  // B
       if (j + 1 == a.nsteps) break;
       __syncthreads();  // A
     }
@@ -221,23 +220,33 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
     if (!failed && rank == 0 && lane == 0) *a.t = t;
     cluster_sync();  // no block pushes any more, and s_sent is complete
     if (failed) {
+      // What may be on its way: of the last two epochs armed, and of a ring's
+      // one after those when the wait that gave up was for RK2's first stage
+      // (the block then still pushed that step, which its neighbours answer).
       bool drained = true;
-#pragma unroll
       for (unsigned b = 0; b < 2; ++b) {
         const unsigned e = armed_ring - b, m = armed_min - b;
-        unsigned missing = 0u;  // bytes of epoch e that were never sent
+        unsigned ahead = 0u;  // bytes of epoch e + 2
         for (int r = lane; r < info.y; r += 32) {
           const int i = __ldg(a.ring_id + info.x + r);
-          if (s_sent[index_ok(i, a.n, a.err) ? i / a.tile : rank].x < e) missing += 16u;
+          const unsigned sent = s_sent[index_ok(i, a.n, a.err) ? i / a.tile : rank].x;
+          if (sent < e) forgo_tx(&ring_bar[e & 1u], 16u);
+          if (sent >= e + 2u) ahead += 16u;
         }
-        missing = __reduce_add_sync(0xffffffffu, missing);
-        if (lane == 0 && missing) forgo_tx(&ring_bar[e & 1u], missing);
-        const unsigned silent = __popc(
-            __ballot_sync(0xffffffffu, lane < blocks && s_sent[lane % kLoopMaxTiles].y <= m));
-        if (lane == 0 && silent) forgo_tx(&min_bar[m & 1u], silent * kWarps * 4u);
+        ahead = __reduce_add_sync(0xffffffffu, ahead);
+        if (lane < blocks && s_sent[lane].y <= m)
+          for (int k = 0; k < kWarps; ++k) forgo_tx(&min_bar[m & 1u], 4u);
         __syncwarp();
-        drained = await(&ring_bar[e & 1u], ((e - 1u) >> 1) & 1u, a.drain_polls) && drained;
-        drained = await(&min_bar[m & 1u], (m >> 1) & 1u, a.drain_polls) && drained;
+        drained = __all_sync(0xffffffffu,
+                             await(&min_bar[m & 1u], (m >> 1) & 1u, a.drain_polls) && drained);
+        if (__all_sync(0xffffffffu,
+                       await(&ring_bar[e & 1u], ((e - 1u) >> 1) & 1u, a.drain_polls))) {
+          if (lane == 0) mbar_expect_tx(&ring_bar[e & 1u], ahead);
+          __syncwarp();
+          drained = await(&ring_bar[e & 1u], ((e + 1u) >> 1) & 1u, a.drain_polls) && drained;
+        } else {
+          drained = false;
+        }
       }
       if (!drained) atomicOr(a.err, 4);
     }
@@ -369,9 +378,8 @@ __global__ void __launch_bounds__(THREADS + 32, 1) k_loop(LoopArgs a) {
     ++epoch;
     if (RK2 || !last) pushed = epoch;
     if (RK2) {
+      __syncthreads();  // B: U* of the tile is complete
       await_ring();
-      stop = __syncthreads_or(fail);  // B: U* of the tile and its ring is complete
-      if (stop) break;
       if (has) {
         fluxes(s1);
         finish(std::integral_constant<int, kModeRK2b>{}, s1, s0, dt, !last);
