@@ -440,7 +440,8 @@ int fv_mesh_debug_set_index(fv_mesh* mesh, int32_t table, int64_t cell, int32_t 
  * (fv_mesh_set_variant) and that step without a closure run the whole loop in
  * one launch on one thread-block cluster instead (also with two steps per
  * launch, when their tile size was left to the library); same bits.  The
- * tables of what the library chooses are built by the first call that runs it.
+ * tables of what the library chooses are built by the first call that runs it
+ * (which synchronises the stream).
  * In a stream that the caller captures, a mesh without a chosen shape steps on
  * shape 0 or 1, whose arrays only fv_renumber and fv_mesh_destroy change: the
  * captured steps stay valid whatever shape is set later. */

@@ -315,6 +315,14 @@ bool capturing(cudaStream_t s) {
   return st != cudaStreamCaptureStatusNone;
 }
 
+// Lets this thread allocate while a stream is captured, by this thread or (a
+// capture in the global mode bars every thread) by another one.
+struct AllocationsAllowed {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  AllocationsAllowed() { FV_CUDA(cudaThreadExchangeStreamCaptureMode(&mode)); }
+  ~AllocationsAllowed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Several host arrays for one device allocation and one copy.
 struct Staging {
   std::vector<unsigned char> host;
@@ -689,6 +697,7 @@ bool uses_loop(const fv_mesh* m, const fv_closure* cl) {
 // holds it.
 void ensure_default(fv_mesh* m, cudaStream_t s) {
   if (m->captured) return;
+  AllocationsAllowed allowed;
   if (wants_loop(m, nullptr)) ensure_loop(m, s);
   if (m->shape_chosen || m->blocking == 2 || uses_loop(m, nullptr)) return;
   if (!m->auto_known) choose_shape(m, s);
@@ -2260,16 +2269,12 @@ void ensure_grad_cells(fv_closure* c, int64_t n, cudaStream_t s) {
       c->cells_outgrown.push_back(c->scratch.cells);
       c->scratch.cells = nullptr;
     }
+    AllocationsAllowed allowed;
     // the stream may still read the smaller array (cudaFree waits for it)
     dev_free(c->scratch.cells);
     c->cells_cap = 0;
     c->cells_captured = false;
-    // an allocation is no part of a capture, but this thread may be barred from it meanwhile
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    if (captured) FV_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
-    const cudaError_t e = cudaMalloc((void**)&c->scratch.cells, n * sizeof(float4));
-    if (captured) cudaThreadExchangeStreamCaptureMode(&mode);
-    FV_CUDA(e);
+    FV_CUDA(cudaMalloc((void**)&c->scratch.cells, n * sizeof(float4)));
     c->cells_cap = n;
   }
   c->cells_captured = c->cells_captured || captured;
