@@ -67,10 +67,11 @@ constexpr int kBatchTile = 1024;  // cells per tile of the batched shared-memory
 // to wait for), steps per launch at most (bounds the time of one launch) and
 // tries of a wait (about a second).  It takes meshes of up to kLoopMaxTiles *
 // kLoopMaxTile = 12,288 cells, one per thread.  Measured (us per step, forward
-// Euler, compensated; shape 1 / tiles of 128 / loop): 1,024 cells 2.4 / 2.5 /
-// 0.93, 4,096 2.8 / 2.5 / 0.99, 8,192 2.8 / 2.5 / 1.5; two cells per thread
-// lose their lead (16,200 cells 2.9 / 2.5 / 2.7, 32,768 2.9 / 2.7 / 4.3): 16
-// SMs then compute longer than a launch on all of them takes.
+// Euler, compensated; shape 1 / one-wave tiles of 128 / loop): 1,024 cells 2.25
+// / 1.77 / 0.79, 4,096 2.36 / 1.81 / 0.86, 8,192 2.27 / 1.81 / 1.18, 12,288 2.54
+// / 1.83 / 1.51.  With two cells per thread a trial of it took 2.7 at 16,200
+// cells and 4.3 at 32,768: 16 SMs then compute longer than a launch on all of
+// them takes.
 constexpr int64_t kLoopMinTile = 64;
 constexpr int64_t kLoopMaxCells = (int64_t)fv::kLoopMaxTiles * fv::kLoopMaxTile;
 constexpr int64_t kLoopSteps = 4096;
@@ -472,9 +473,9 @@ int sm_count() {
 // Tiles of shape 7 in FP64: as few as fit, the same number on every SM and all
 // of one size (an SM with one tile more holds the others up), of up to 1,700
 // cells (some 200 KB of shared memory): large tiles have short rings.  us per
-// step with 1 / 2 / 4 tiles per SM: 12,800 cells 6.6 / 6.9 / 8.3, 102,400
-// 22.6 / 23.1 / 24.7, 250,000 47.4 / 48.6 / 49.7; 640,000 with 3 / 4 / 8: 118 /
-// 124 / 121.
+// step with 1 / 2 / 4 tiles per SM: 12,800 cells 6.3 / 6.6 / -, 102,400 21.6 /
+// 22.1 / 23.6, 250,000 43.6 / 44.8 / 45.9; 640,000 with 3 / 4 / 8: 112 / 118 /
+// 113.
 int64_t fp64_tile(int64_t n) {
   const int64_t sms = sm_count(), per_sm = (n + sms - 1) / sms;
   const int64_t tiles = (per_sm + 1699) / 1700;
@@ -587,15 +588,18 @@ bool leaves_memory(size_t bytes) {
 }
 
 // The step-kernel shape of a mesh whose shape was not chosen, by size
-// (measured us per step, forward Euler):
-//   FP64: shape 7 (102,400 cells: 24.5 against 52 for shape 1; 12,800: 9.4
-//   against 19.2), whose tiles must be compact: with rings of more than 2.5
+// (measured us per step on the periodic square, forward Euler, FP32
+// compensated):
+//   FP64: shape 7 (102,400 cells: 21.6 against 51 for shape 1; 12,800: 6.3
+//   against 18.3), whose tiles must be compact: with rings of more than 2.5
 //   times the tile a face evaluated once no longer pays for staging the ring;
 //   else shape 1, which needs no tables;
-//   FP32: up to 90,000 cells the one-wave tiles (65,536: 2.4 against 2.6 for
-//   shape 0, 102,400: 3.1 against 2.8) when their rings hold less than 3/4 of
-//   the cells, then shape 0 (160,000: 3.5 against 3.9 for shape 1) up to
-//   230,000 (250,000: 5.3 against 4.8), then shape 1.
+//   FP32: up to 90,000 cells the one-wave tiles (65,536: 2.22 against 2.50 for
+//   shape 0, 102,400: 3.16 against 3.00) when their rings hold less than 3/4 of
+//   the cells, then shape 0 (160,000: 3.84 against 4.04 for shape 1) up to
+//   230,000 (250,000: 5.27 against 4.93), then shape 1.  (Above 77,824 cells,
+//   four tiles of 128 an SM, the tiles are of 160, and the line could lie there:
+//   89,600: 3.26 against 2.94 for shape 0.)
 void choose_shape(fv_mesh* m, cudaStream_t s) {
   const int64_t n = m->h.n;
   m->auto_variant = m->plain_shape();

@@ -10,7 +10,7 @@
 // The one-wave tile kernel also signals `griddepcontrol.launch_dependents`
 // (chain_next) right after that wait, so that the next grid's blocks start
 // beside its own and read their tables while it computes: 65,536 cells on
-// tiles of 128 take 2.4 us per step, against 3.2 without.  (Signalled before the
+// tiles of 128 take 2.5 us per step, against 3.2 without.  (Signalled before the
 // wait, several grids queue up on the SMs and spread the running one unevenly:
 // 3.2 us.)  Elsewhere the signal costs more than it hides: the persistent
 // shape 1 ran 5-10 % slower on 160,000 to 1M cells (4.07 -> 4.65, 9.2 -> 9.8 us),

@@ -380,8 +380,8 @@ __device__ __forceinline__ bool rough_bound(const dq4& U, double inradius, float
 // 64 clocks): the tile's tables and each thread's first face are read before
 // the previous step ends, the blocks have about a thread per face, and one more
 // warp forms dt.
-// Measured (us per step): channel of 250,000 cells, autotuned, 88 -> 45;
-// square of 12,800 cells 19.2 (shape 1) -> 6.5.
+// Measured (us per step): channel of 250,000 cells, autotuned, 89 -> 46;
+// square of 12,800 cells 18.3 (shape 1) -> 6.3.
 template <int MODE, int THREADS, int KMAX, int WAVE>
 __global__ void __launch_bounds__(THREADS + 32) k_step_faces64(StepArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
