@@ -359,8 +359,9 @@ def run_ours(args):
                     + " + k_step_scaled")
         else:
             kfun = {5: "k_step_tma", 6: "k_step_tile",
-                    7: "k_step_faces64" if prec == "f64" else "k_step_tile_faces"}.get(
-                tune["variant"], "k_step")
+                    7: "k_step_faces64" if prec == "f64" else "k_step_tile_faces",
+                    B.KERNEL_LOOP: "k_loop", B.KERNEL_ONE_WAVE: "k_step_tile_quick"}.get(
+                m.step_kernel()[0], "k_step")
         kname = (f"{kfun}<{'float' if prec == 'f32' else 'double'}, "
                  f"{'RK2' if stages == 2 else 'FE'}, "
                  f"{'compensated' if comp else 'plain'}, shape {tune['variant']}"
@@ -408,7 +409,10 @@ def run_ours(args):
                          else f"step_{prec}{'' if comp or prec == 'f64' else '_plain'}"
                               f"_{args.workload}.md")},
         "e2e": e2e,
-        "gpu_launches": args.steps * (launches + 3),
+        # the loop's scalars, its first bound, its steps and the totals; the resident
+        # loop has its bound inside and takes 4096 steps a launch
+        "gpu_launches": args.steps * (-(-S // 4096) + 2 if m.step_kernel()[0] == B.KERNEL_LOOP
+                                      else launches + 3),
         "clocks": clk.summary(),
     }
     if rank == 0 and not args.no_extras and world == 1:
@@ -480,7 +484,7 @@ def run_batch(args, B, spec, dist, world, rank):
         t = torch.tensor([total], device="cuda", dtype=torch.float64)
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
         total = float(t.item())
-    shape = batch.variant()
+    shape = batch.step_kernel()
     avg_launch = total / (args.steps * S)
     peak, peak_kind = measured_peaks()
     kbytes = ALGO_BYTES[prec] + (COMP_BYTES if update == "compensated" else 0)
