@@ -21,6 +21,7 @@
 // the same tile, the face of that neighbour that points back (the tile
 // kernel that evaluates each face once writes the negated flux there).
 #include <algorithm>
+#include <cmath>
 #include <exception>
 #include <functional>
 #include <thread>
@@ -150,20 +151,56 @@ struct TilePart {
   int32_t t1_cap = 0, f_cap = 0;
 };
 
+// The cells of one tile's ring at a time and their places in it: an open table
+// whose entries of earlier tiles are told by their stamp.
+class RingTable {
+ public:
+  explicit RingTable(int32_t tile) {
+    int bits = 4;
+    while (((int64_t)1 << bits) < 8 * (int64_t)tile) ++bits;  // three neighbours a cell at most
+    shift_ = 32 - bits;
+    slots_.resize((size_t)1 << bits);
+  }
+  void next_tile() { ++now_; }
+  // The place of cell x; `fresh` where it was not there (its place is then unset).
+  int32_t& at(int32_t x, bool& fresh) {
+    const uint32_t mask = (uint32_t)slots_.size() - 1u;
+    uint32_t k = ((uint32_t)x * 2654435761u) >> shift_;
+    while (slots_[k].stamp == now_ && slots_[k].cell != x) k = (k + 1u) & mask;
+    fresh = slots_[k].stamp != now_;
+    if (fresh) slots_[k] = Slot{x, 0, now_};
+    return slots_[k].place;
+  }
+
+ private:
+  struct Slot {
+    int32_t cell = 0, place = 0;
+    int64_t stamp = -1;
+  };
+  std::vector<Slot> slots_;
+  int shift_;
+  int64_t now_ = 0;
+};
+
 void step_tile_range(const HostMesh& m, int32_t tile, bool faces, int32_t b0, int32_t b1,
                      PairTiles& L, TilePart& part) {
   std::vector<int32_t> ring;
   std::vector<uint32_t> ghosts;
+  RingTable places((int32_t)std::min<int64_t>(tile, m.n));
+  bool fresh = false;
   for (int32_t b = b0; b < b1; ++b) {
     const int64_t t0 = (int64_t)b * tile, t1 = std::min<int64_t>(t0 + tile, m.n);
     const int32_t nt = (int32_t)(t1 - t0);
     ring.clear();
+    places.next_tile();
     for (int64_t j = 3 * t0; j < 3 * t1; ++j) {
       const int32_t x = m.nbr[j];
-      if (x >= 0 && (x < t0 || x >= t1)) ring.push_back(x);
+      if (x < 0 || (x >= t0 && x < t1)) continue;
+      places.at(x, fresh);
+      if (fresh) ring.push_back(x);
     }
     std::sort(ring.begin(), ring.end());
-    ring.erase(std::unique(ring.begin(), ring.end()), ring.end());
+    for (size_t e = 0; e < ring.size(); ++e) places.at(ring[e], fresh) = nt + (int32_t)e;
     if (nt + (int64_t)ring.size() > kLocalLimit)
       throw Error{FV_EINVAL, "a tile with its halo exceeds 65533 cells; renumber the cells "
                              "with a compact order (Hilbert) or use smaller tiles"};
@@ -179,7 +216,7 @@ void step_tile_range(const HostMesh& m, int32_t tile, bool faces, int32_t b0, in
         if (x < 0) {
           v[k] = (uint32_t)(0x10000 + x);
         } else if (x < t0 || x >= t1) {
-          v[k] = (uint32_t)(nt + (std::lower_bound(ring.begin(), ring.end(), x) - ring.begin()));
+          v[k] = (uint32_t)places.at(x, fresh);
         } else {
           v[k] = (uint32_t)(x - t0);
           if (!faces) continue;
@@ -260,7 +297,10 @@ PairTiles build_step_tiles(const HostMesh& m, int32_t tile, bool faces) {
   L.tile_info.assign(2 * (L.n_tiles + 1), 0);
   L.cell_ln.resize(2 * (size_t)m.n);
   if (faces) L.cell_ref.assign(2 * (size_t)m.n, 0u);
-  const int workers = host_workers(m.n);
+  // starting a thread takes some 50 us, a cell some 10 ns: the time falls until
+  // the square root of their ratio (host_workers' many threads spent 0.8 ms on
+  // being started for 60,000 cells)
+  const int workers = std::min(host_workers(m.n), 1 + (int)std::sqrt((double)m.n / 5000.0));
   std::vector<TilePart> parts(workers);
   on_host_threads(workers, [&](int w) {
     step_tile_range(m, tile, faces, (int32_t)(L.n_tiles * w / workers),
