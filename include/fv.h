@@ -577,7 +577,7 @@ int fv_batch_info(const fv_batch* batch, int64_t* n_cells_padded, int64_t* offse
  * memory (needs compactly numbered meshes: FV_EINVAL if a tile's ring does
  * not fit).  Default: 6 when its tiles fit, else 0 (decided at the first
  * device call); until a shape is set the steps run whichever of 0 and 6 is
- * quicker for the batch's precision and size.  All give bitwise identical
+ * quicker for the batch's precision, update and size.  All give bitwise identical
  * results. */
 int fv_batch_set_variant(fv_batch* batch, int32_t variant);
 

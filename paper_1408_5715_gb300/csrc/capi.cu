@@ -1707,11 +1707,20 @@ struct fv_batch {
   bool compensated = true;
   // 0: one thread per cell; 5: TMA-staged tiles; 6: tiles; -1: 6 when its
   // tiles fit in shared memory, else 0 (at the first device call).  While none
-  // was chosen the steps run the quicker of 0 and 6 (auto_variant).
+  // was chosen the steps run the quicker of 0 and 6 (auto_shape).
   int variant = -1;
   bool shape_chosen = false;
-  int auto_variant = 0;
-  int shape() const { return shape_chosen ? variant : auto_variant; }
+  int shape() const { return shape_chosen ? variant : auto_shape(); }
+  // us per step, shape 0 / 6, forward Euler: FP32 plain 96,024 cells 3.4 / 5.3,
+  // 1,046,024 14.3 / 19.0, 2,457,668 39.7 / 45.5, 5,083,648 78 / 82; compensated
+  // (whose remainder is read and written where the cells' records are) 3.6 / 5.4,
+  // 16.3 / 17.6, 44.1 / 43.3, 86.5 / 87.0, and with RK2 35.4 / 36.9, 100 / 95, 200 /
+  // 191; FP64 70,124 36 / 57, 307,332 137 / 123 (few large tiles idle most SMs of a
+  // small FP64 batch, while on a large one forming every primitive four times
+  // costs more)
+  int auto_shape() const {
+    return (f64() && n > 200000) || (use_lo() && n > 2000000) ? variant : 0;
+  }
   int ran_kernel = FV_KERNEL_NONE;  // fv_batch_get_step_kernel
   // shared-memory tiles of 1024 cells within each mesh (shape 6)
   bool tiles_ok = false;
@@ -1878,11 +1887,6 @@ void batch_ensure_device(fv_batch* b, cudaStream_t s) {
     const bool fits =
         b->tiles_ok && fv::tile_smem_bytes(b->f64(), b->t1_cap) <= (size_t)optin;
     b->variant = fits ? fv::kTileVariant : 0;
-    // us per step, shape 0 / 6: FP32 18,056 cells 3.3 / 5.4, 307,332 6.7 / 7.7,
-    // 2,457,668 plain 39.5 / 45.4, compensated 43.7 / 43.2; FP64 70,124 36 / 57,
-    // 307,332 137 / 123 (few large tiles idle most SMs of a small FP64 batch,
-    // while on a large one forming every primitive four times costs more)
-    b->auto_variant = b->f64() && n > 200000 ? b->variant : 0;
   }
 }
 
