@@ -522,7 +522,9 @@ int fv_mesh_set_closure_engine(fv_mesh* mesh, int32_t engine);
  * weights: host double[4] (> 0).  loss: host double (nullable; if given, the
  * stream is synchronised).  grad: device FP32 [1377] dL/dtheta in the order of
  * fv_closure_create (nullable), differentiated through the bfloat16 roundings
- * as if they were the identity.  Deterministic (fixed reduction order). */
+ * as if they were the identity.  Deterministic (fixed reduction order).
+ * Without a loss the call may be captured into a graph, which may be replayed
+ * until the closure or the mesh is destroyed or the mesh renumbered. */
 int fv_closure_loss_grad(fv_mesh* mesh, const void* U0, const void* Ut, double dt,
                          const double* weights, fv_closure* closure, double* loss, float* grad,
                          void* stream);

@@ -606,8 +606,8 @@ void choose_shape(fv_mesh* m, cudaStream_t s) {
   m->auto_tile = 0;
   if (!m->f64() && n > 90000) return;
   const int tile = (int)(m->f64() ? fp64_tile(n) : quick_tile(n));
-  bool good = m->f64() ? leaves_memory(fp64_table_bytes(n)) : true;
-  good = good && optional_tables([&] {
+  const bool good = optional_tables([&] {
+    if (m->f64() && !leaves_memory(fp64_table_bytes(n))) invalid("little memory left for tables");
     fv::PairTiles L = fv::build_step_tiles(m->h, tile, m->f64());
     const int64_t rings = (int64_t)L.halo_id.size();
     if (m->f64() ? 2 * rings > 5 * n
