@@ -2311,6 +2311,8 @@ int fv_closure_create(const float* theta, fv_closure** out) {
       FV_CUDA(cudaMalloc((void**)&t.lpart, (size_t)t.loss_blocks * sizeof(double)));
       FV_CUDA(cudaMalloc((void**)&c->d_grad, fv::kClosureParams * sizeof(float)));
       FV_CUDA(cudaMalloc((void**)&t.loss, sizeof(double)));
+      FV_CUDA(cudaMalloc((void**)&t.gmax, 2 * sizeof(unsigned)));
+      FV_CUDA(cudaMemset(t.gmax, 0, 2 * sizeof(unsigned)));
       closure_upload(c, theta, false, nullptr);
     } catch (...) {
       cudaFree(c->d_w1);
@@ -2321,6 +2323,7 @@ int fv_closure_create(const float* theta, fv_closure** out) {
       cudaFree(c->scratch.lpart);
       cudaFree(c->d_grad);
       cudaFree(c->scratch.loss);
+      cudaFree(c->scratch.gmax);
       delete c;
       throw;
     }
@@ -2342,6 +2345,7 @@ int fv_closure_destroy(fv_closure* closure) {
     cudaFree(closure->scratch.lpart);
     cudaFree(closure->d_grad);
     cudaFree(closure->scratch.loss);
+    cudaFree(closure->scratch.gmax);
     delete closure;
   });
 }

@@ -978,8 +978,9 @@ unsigned cl_grid(K kernel, int64_t items_per_warp_group, int64_t n) {
 // is added to FP32 accumulators in registers (the tensor core's own
 // accumulation rounds toward zero: chained over the three parts of a tile its
 // bias made the gradient's error 2.4e-7, against 1.2e-7 this way and 1.5e-7 for
-// the former row-by-row sums).  Below 2^-109 the third part sinks under
-// bfloat16's smallest values and an operand keeps fewer bits.
+// the former row-by-row sums).  Below 2^-109 the third part would sink under
+// bfloat16's smallest values, so G enters with its largest magnitude brought to
+// 1..2 by a power of two, which the final sums take out again (both exact).
 // Measured on 250,000 cells: 275 us for the former row-by-row backward (lane o
 // a unit, 64 shuffles and shared-memory reads per row, every face from both
 // sides) against 27 + 44 us (ncu); a training iteration (loss, gradient, Adam,
@@ -993,7 +994,8 @@ __device__ __forceinline__ float bf16_hi(unsigned v) { return __uint_as_float(v 
 
 __global__ void __launch_bounds__(kClThreads) k_closure_cells(StepArgs a, const float4* Ut, float dt,
                                                               float4 wq, ClosureParams cp,
-                                                              float4* G, double* lpart) {
+                                                              float4* G, double* lpart,
+                                                              unsigned* gmax) {
   __shared__ ClShared sh;
   load_small_params(cp, sh);
   ClFrag fr;
@@ -1005,6 +1007,7 @@ __global__ void __launch_bounds__(kClThreads) k_closure_cells(StepArgs a, const 
   const float iw2[4] = {1.0f / (wq.x * wq.x), 1.0f / (wq.y * wq.y), 1.0f / (wq.z * wq.z),
                         1.0f / (wq.w * wq.w)};
   double loss = 0.0;
+  unsigned largest = 0u;  // bits of the largest |G|
   const int n = (int)a.n;
   const int wstride = gridDim.x * kClWarps * 32;
   for (int base = (blockIdx.x * kClWarps + warp) * 32; base < n; base += wstride) {
@@ -1052,20 +1055,31 @@ __global__ void __launch_bounds__(kClThreads) k_closure_cells(StepArgs a, const 
       for (int q = 0; q < 4; ++q) {
         loss += (double)V * (double)d[q] * (double)d[q] * (double)iw2[q];
         g[q] = 2.0f * V * d[q] * iw2[q] * f;
+        largest = max(largest, __float_as_uint(g[q]) & 0x7fffffffu);
       }
       G[i] = make_float4(g[0], g[1], g[2], g[3]);
     }
     __syncwarp();
   }
   for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
+  largest = __reduce_max_sync(0xffffffffu, largest);
   __shared__ double lw[kClWarps];
-  if (lane == 0) lw[warp] = loss;
+  __shared__ unsigned gw[kClWarps];
+  if (lane == 0) lw[warp] = loss, gw[warp] = largest;
   __syncthreads();
   if (threadIdx.x == 0) {
     double l = 0.0;
-    for (int wv = 0; wv < kClWarps; ++wv) l += lw[wv];
+    for (int wv = 0; wv < kClWarps; ++wv) l += lw[wv], largest = max(largest, gw[wv]);
     lpart[blockIdx.x] = l;
+    atomicMax(gmax, largest);
   }
+}
+
+// The exponent field of the power of two that brings the largest |G| to 1..2
+// (for 0 and non-finite ones: none), within the normal floats.
+__device__ __forceinline__ int grad_exponent(unsigned largest) {
+  if (largest == 0u || largest >= 0x7f800000u) return 127;
+  return min(max((int)(largest >> 23), 1), 253);
 }
 
 // Transpose of an 8 x 8 matrix of 16-bit values held one row pair per lane.
@@ -1095,6 +1109,7 @@ struct GrShared {
   // (W2[k][n]), for the K slices 0 (x, y) and 1 (z, w)
   uint4 w2[4][32], w2t[4][32];
   float w3[32];
+  float up;  // the power of two that G is scaled by
   union {
     GrWarpSmem warp[kGrWarps];
     float red[kGrWarps][kClosureParams];  // the block's gradients, at the end
@@ -1218,8 +1233,14 @@ __device__ __forceinline__ void grad_tile(const GrShared& sh, const GrWarpSmem& 
 
 __global__ void __launch_bounds__(kGrThreads, 3) k_closure_grad(StepArgs a,
                                                                 const float4* __restrict__ G,
-                                                                ClosureParams cp, float* gpart) {
+                                                                ClosureParams cp, float* gpart,
+                                                                unsigned* gmax) {
   __shared__ GrShared sh;
+  if (threadIdx.x == 0) {
+    const unsigned largest = gmax[0];
+    sh.up = __uint_as_float((unsigned)(254 - grad_exponent(largest)) << 23);
+    if (blockIdx.x == 0) gmax[1] = largest;  // for the final sums
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = lane >> 2, cq = lane & 3;
   ClFrag fr;
   load_frags(cp, fr);
@@ -1279,8 +1300,11 @@ __global__ void __launch_bounds__(kGrThreads, 3) k_closure_grad(StepArgs a,
         const float qL = fma_(L.u, nx[k], mul(L.v, ny[k]));
         const float qR = fma_(W.u, nx[k], mul(W.v, ny[k]));
         const float na = mul(-0.25f, fma_(len, add(L.c, W.c), fabsf(add(qL, qR))));
-        w.gs[at] = (Gi.x - Gb.x) * (na * (UR.x - c.U.x)) + (Gi.y - Gb.y) * (na * (UR.y - c.U.y)) +
-                   (Gi.z - Gb.z) * (na * (UR.z - c.U.z)) + (Gi.w - Gb.w) * (na * (UR.w - c.U.w));
+        const float up = sh.up;
+        w.gs[at] = up * (Gi.x - Gb.x) * (na * (UR.x - c.U.x)) +
+                   up * (Gi.y - Gb.y) * (na * (UR.y - c.U.y)) +
+                   up * (Gi.z - Gb.z) * (na * (UR.z - c.U.z)) +
+                   up * (Gi.w - Gb.w) * (na * (UR.w - c.U.w));
       }
       rows += __popc(who);
     }
@@ -1347,7 +1371,8 @@ __global__ void __launch_bounds__(kGrThreads, 3) k_closure_grad(StepArgs a,
 // threads each over every eighth partial; the last block sums the loss.
 __global__ void __launch_bounds__(256) k_closure_grad_final(const float* gpart, int nblocks,
                                                             const double* lpart, int lblocks,
-                                                            float* grad, double* loss) {
+                                                            float* grad, double* loss,
+                                                            unsigned* gmax) {
   __shared__ double sm[256];
   const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
   double s = 0.0;
@@ -1358,7 +1383,10 @@ __global__ void __launch_bounds__(256) k_closure_grad_final(const float* gpart, 
     if (threadIdx.x < 32) {
       for (int k = 1; k < 8; ++k) s += sm[32 * k + lane];
       for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-      if (lane == 0) *loss = s;
+      if (lane == 0) {
+        *loss = s;
+        gmax[0] = 0u;  // at rest for the next call
+      }
     }
     return;
   }
@@ -1369,7 +1397,8 @@ __global__ void __launch_bounds__(256) k_closure_grad_final(const float* gpart, 
   __syncthreads();
   if (slice == 0 && j < kClosureParams) {
     for (int k = 1; k < 8; ++k) s += sm[32 * k + lane];
-    grad[j] = (float)s;
+    // times 2^(exponent - 127)
+    grad[j] = (float)(s * __hiloint2double((grad_exponent(gmax[1]) - 127 + 1023) << 20, 0));
   }
 }
 
@@ -1450,10 +1479,10 @@ cudaError_t launch_closure_grad(const StepArgs& a, const float* Ut, double dt, c
   k_closure_cells<<<lb, kClThreads, 0, s>>>(a, reinterpret_cast<const float4*>(Ut), (float)dt,
                                             make_float4((float)w[0], (float)w[1], (float)w[2],
                                                         (float)w[3]),
-                                            cp, sc.cells, sc.lpart);
-  k_closure_grad<<<gb, kGrThreads, 0, s>>>(a, sc.cells, cp, sc.gpart);
+                                            cp, sc.cells, sc.lpart, sc.gmax);
+  k_closure_grad<<<gb, kGrThreads, 0, s>>>(a, sc.cells, cp, sc.gpart, sc.gmax);
   k_closure_grad_final<<<(kClosureParams + 31) / 32 + 1, 256, 0, s>>>(sc.gpart, gb, sc.lpart, lb,
-                                                                      grad, sc.loss);
+                                                                      grad, sc.loss, sc.gmax);
   return cudaGetLastError();
 }
 

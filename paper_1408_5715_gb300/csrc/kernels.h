@@ -177,6 +177,7 @@ struct ClosureScratch {
   float* gpart;   // [grad_blocks * kClosureParams]
   double* lpart;  // [loss_blocks]
   double* loss;   // [1], written
+  unsigned* gmax;  // [2] the largest |cells| (bits; [0] is 0 between calls)
   int grad_blocks, loss_blocks;
 };
 // One-step loss and gradient (grad: [kClosureParams], written).
